@@ -101,8 +101,9 @@ struct bacon_ctx {
     void* hvo_buf = nullptr;
     int32_t* hidx_buf = nullptr;
     size_t hq_cap = 0, hk_cap = 0, hv_cap = 0, hko_cap = 0, hvo_cap = 0, hidx_cap = 0;
-    // TMA descriptors of the last whole-step call: [kMaxPairs] K maps, then
-    // [kMaxPairs] window-query maps (device copy + pinned host staging)
+    // TMA descriptors of the last whole-step call on unevenly spaced tensors:
+    // [kMaxPairs] K maps, then [kMaxPairs] window-query maps (device copy +
+    // pinned host staging)
     CUtensorMap* d_maps = nullptr;
     CUtensorMap* h_maps = nullptr;
     cudaEvent_t maps_ev = nullptr;
@@ -135,11 +136,6 @@ struct bacon_state {
     float* lam = nullptr;
     float* lse2 = nullptr;
     float2* partial = nullptr;
-    CUtensorMap* d_maps = nullptr;  // [0] K map, [1] window-query map
-    CUtensorMap* h_maps = nullptr;
-    cudaEvent_t maps_ev = nullptr;
-    std::vector<const void*> map_key;
-    int map_key_N = -1;
 };
 
 namespace {
@@ -185,18 +181,52 @@ bacon_status check_seq(const bacon_ctx* c, int N, int budget)
     return BACON_OK;
 }
 
-// Encode the TMA descriptors of the (request, layer) pairs in slots
-// [map0, map0 + pairs) and copy them to `d_maps` on the stream (K maps at
-// [0, stride), query maps at [stride, 2 stride)); skipped when those slots
-// already hold the same pointers for this N.
-bacon_status upload_maps(const bacon_ctx* c, CUtensorMap* d_maps, CUtensorMap* h_maps,
-                         cudaEvent_t ev, std::vector<const void*>& key, int& key_N, int stride,
-                         int map0, int pairs, const void* const* q, const void* const* k, int N,
-                         cudaStream_t st)
+// The distance in bytes between consecutive pairs' tensors when it is the
+// same for all of them and one TMA descriptor can span it: a positive
+// multiple of the row's bytes that a block of `rows` rows does not exceed,
+// below the descriptor's 2^40 limit.  0 when there is none.
+long long pair_spacing(const void* const* p, int pairs, long long rows, int d)
 {
-    if (key_N != N || (int)key.size() != 2 * stride) {
+    const long long row = 2LL * d, block = rows * row;
+    if (pairs == 1) return block;
+    // compared as integers: the tensors may be separate allocations
+    const uintptr_t p0 = reinterpret_cast<uintptr_t>(p[0]), p1 = reinterpret_cast<uintptr_t>(p[1]);
+    if (p1 <= p0 || p1 - p0 >= ((uintptr_t)1 << 40)) return 0;
+    const long long step = (long long)(p1 - p0);
+    if (step < block || step % row) return 0;
+    for (int i = 2; i < pairs; ++i)
+        if (reinterpret_cast<uintptr_t>(p[i]) != p0 + (uintptr_t)step * i) return 0;
+    return step;
+}
+
+// One TMA descriptor over every pair's K and one over every pair's window
+// queries, as kernel parameters; false when the tensors are not evenly
+// spaced (or the encoding is refused), and the table of one map per pair is
+// needed.
+bool bind_maps(const bacon_ctx* c, TcMaps& m, int pairs, const void* const* q,
+               const void* const* k, int N)
+{
+    const long long krows = (long long)c->hkv * N, qrows = (long long)c->hq * c->W;
+    const long long ks = pair_spacing(k, pairs, krows, c->d), qs = pair_spacing(q, pairs, qrows, c->d);
+    return ks && qs && encode_rows_map(&m.k, k[0], c->d, krows, pairs, ks, kTcKBoxRows) &&
+           encode_rows_map(&m.q, q[0], c->d, qrows, pairs, qs, kTcQBoxRows);
+}
+
+// Encode one TMA descriptor per (request, layer) pair in slots
+// [map0, map0 + pairs) and copy them to the context's device table on the
+// stream (K maps at [0, kMaxPairs), query maps behind them); skipped when
+// those slots already hold the same pointers for this N.
+bacon_status upload_maps(bacon_ctx* c, int map0, int pairs, const void* const* q,
+                         const void* const* k, int N, cudaStream_t st)
+{
+    CUtensorMap* const d_maps = c->d_maps;
+    CUtensorMap* const h_maps = c->h_maps;
+    const cudaEvent_t ev = c->maps_ev;
+    std::vector<const void*>& key = c->map_key;
+    constexpr int stride = kMaxPairs;
+    if (c->map_key_N != N || (int)key.size() != 2 * stride) {
         key.assign(2 * stride, nullptr);  // every slot must be encoded again
-        key_N = N;
+        c->map_key_N = N;
     }
     bool same = true;
     for (int i = 0; same && i < pairs; ++i)
@@ -204,8 +234,10 @@ bacon_status upload_maps(const bacon_ctx* c, CUtensorMap* d_maps, CUtensorMap* h
     if (same) return BACON_OK;
     BACON_CUDA(cudaEventSynchronize(ev), "descriptor staging wait");
     for (int i = 0; i < pairs; ++i) {
-        if (!encode_rows_map(h_maps + map0 + i, k[i], c->d, (long long)c->hkv * N, kTcKBoxRows) ||
-            !encode_rows_map(h_maps + stride + map0 + i, q[i], c->d, (long long)c->hq * c->W,
+        const long long krows = (long long)c->hkv * N, qrows = (long long)c->hq * c->W;
+        if (!encode_rows_map(h_maps + map0 + i, k[i], c->d, krows, 1, krows * c->d * 2,
+                             kTcKBoxRows) ||
+            !encode_rows_map(h_maps + stride + map0 + i, q[i], c->d, qrows, 1, qrows * c->d * 2,
                              kTcQBoxRows))
             return fail(BACON_ECUDA, "cuTensorMapEncodeTiled failed for pair %d", map0 + i);
     }
@@ -223,12 +255,11 @@ bacon_status upload_maps(const bacon_ctx* c, CUtensorMap* d_maps, CUtensorMap* h
     return BACON_OK;
 }
 
-TcArgs tc_args(const Shape& s, const CUtensorMap* kmaps, const CUtensorMap* qmaps,
-               float2* partial, const float* lse2, float* B, float* Q, float* E, int* err)
+TcArgs tc_args(const Shape& s, float2* partial, const float* lse2, float* B, float* Q, float* E,
+               int* err)
 {
     TcArgs a;
-    a.kmaps = kmaps;
-    a.qmaps = qmaps;
+    a.kmaps = a.qmaps = nullptr;
     a.s = s;
     a.chunks = (s.N + kTcChunkTokens - 1) / kTcChunkTokens;
     a.total_chunks = s.units * a.chunks;
@@ -333,11 +364,15 @@ bacon_status window_passes(bacon_ctx* c, const Shape& s, const void* const* q,
     const int chunks = (N + kTcChunkTokens - 1) / kTcChunkTokens;
     float* lse2 = c->lse2 + unit0 * c->rows;
     float2* partial = c->partial + unit0 * chunks * c->rows;
-    bacon_status rc = upload_maps(c, c->d_maps, c->h_maps, c->maps_ev, c->map_key, c->map_key_N,
-                                  kMaxPairs, map0, pairs, q, k, N, st);
-    if (rc != BACON_OK) return rc;
-    TcArgs ta = tc_args(s, c->d_maps + map0, c->d_maps + kMaxPairs + map0, partial, lse2,
-                        c->B + unit0 * N, c->Q + unit0 * N, c->E + unit0 * N, c->err);
+    TcArgs ta = tc_args(s, partial, lse2, c->B + unit0 * N, c->Q + unit0 * N, c->E + unit0 * N,
+                        c->err);
+    TcMaps tm;
+    if (!bind_maps(c, tm, pairs, q, k, N)) {
+        bacon_status rc = upload_maps(c, map0, pairs, q, k, N, st);
+        if (rc != BACON_OK) return rc;
+        ta.kmaps = c->d_maps + map0;
+        ta.qmaps = c->d_maps + kMaxPairs + map0;
+    }
     prof.mark(0);
     if (!prefill_lse && window_onepass_fits(s)) {
         // the unit's logits stay in tensor memory: one kernel, one pass over K
@@ -346,7 +381,7 @@ bacon_status window_passes(bacon_ctx* c, const Shape& s, const void* const* q,
         prof.mark(2);
         prof.skip(0);
         prof.skip(1);
-        BACON_CUDA(launch_window_onepass(ta, st), "window_onepass launch");
+        BACON_CUDA(launch_window_onepass(ta, tm, st), "window_onepass launch");
         prof.mark(3);
         return BACON_OK;
     }
@@ -361,15 +396,15 @@ bacon_status window_passes(bacon_ctx* c, const Shape& s, const void* const* q,
             TcArgs tf = ta;
             tf.fault = 1;
             c->fault_pending = 0;
-            BACON_CUDA(launch_window_stats_tc(tf, st), "window_stats launch");
+            BACON_CUDA(launch_window_stats_tc(tf, tm, st), "window_stats launch");
         } else {
-            BACON_CUDA(launch_window_stats_tc(ta, st), "window_stats launch");
+            BACON_CUDA(launch_window_stats_tc(ta, tm, st), "window_stats launch");
         }
         prof.mark(1);
         BACON_CUDA(launch_window_combine(s, ta.chunks, partial, lse2, st), "window_combine launch");
     }
     prof.mark(2);
-    BACON_CUDA(launch_window_scores_tc(ta, st), "window_scores launch");
+    BACON_CUDA(launch_window_scores_tc(ta, tm, st), "window_scores launch");
     prof.mark(3);
     return BACON_OK;
 }
@@ -676,11 +711,6 @@ bacon_status bacon_state_create(bacon_ctx* ctx, bacon_state** out)
     if (e == cudaSuccess) e = dalloc(&st->lam, ctx->hkv);
     if (e == cudaSuccess) e = dalloc(&st->lse2, (size_t)ctx->hkv * ctx->rows);
     if (e == cudaSuccess) e = dalloc(&st->partial, (size_t)ctx->hkv * chunks * ctx->rows);
-    if (e == cudaSuccess) e = dalloc(&st->d_maps, 2);
-    if (e == cudaSuccess)
-        e = cudaHostAlloc(reinterpret_cast<void**>(&st->h_maps), 2 * sizeof(CUtensorMap),
-                          cudaHostAllocDefault);
-    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&st->maps_ev, cudaEventDisableTiming);
     if (e != cudaSuccess) {
         cudaGetLastError();
         bacon_state_destroy(st);
@@ -702,11 +732,9 @@ bacon_status bacon_state_reset(bacon_state* st)
 void bacon_state_destroy(bacon_state* st)
 {
     if (!st) return;
-    void* bufs[] = {st->Ering, st->B, st->Q, st->S, st->lam, st->lse2, st->partial, st->d_maps};
+    void* bufs[] = {st->Ering, st->B, st->Q, st->S, st->lam, st->lse2, st->partial};
     for (void* b : bufs)
         if (b) cudaFree(b);
-    if (st->h_maps) cudaFreeHost(st->h_maps);
-    if (st->maps_ev) cudaEventDestroy(st->maps_ev);
     delete st;
 }
 
@@ -730,14 +758,13 @@ bacon_status bacon_score_layer(bacon_ctx* ctx, bacon_state* st, int layer, const
 
     const Shape s = shape_of(ctx, 1, 1, seq_len);
     float* Eslot = st->Ering + (size_t)(layer % st->ring) * ctx->hkv * seq_len;
-    rc = upload_maps(ctx, st->d_maps, st->h_maps, st->maps_ev, st->map_key, st->map_key_N, 1, 0, 1,
-                     &q_win, &k, seq_len, cs);
-    if (rc != BACON_OK) return rc;
-    const TcArgs ta = tc_args(s, st->d_maps, st->d_maps + 1, st->partial, st->lse2, st->B, st->Q,
-                              Eslot, ctx->err);
-    BACON_CUDA(launch_window_stats_tc(ta, cs), "window_stats launch");
+    TcArgs ta = tc_args(s, st->partial, st->lse2, st->B, st->Q, Eslot, ctx->err);
+    TcMaps tm;
+    if (!bind_maps(ctx, tm, 1, &q_win, &k, seq_len))
+        return fail(BACON_ECUDA, "cuTensorMapEncodeTiled failed");
+    BACON_CUDA(launch_window_stats_tc(ta, tm, cs), "window_stats launch");
     BACON_CUDA(launch_window_combine(s, ta.chunks, st->partial, st->lse2, cs), "window_combine launch");
-    BACON_CUDA(launch_window_scores_tc(ta, cs), "window_scores launch");
+    BACON_CUDA(launch_window_scores_tc(ta, tm, cs), "window_scores launch");
 
     CalibArgs a;
     a.B = st->B;
@@ -1044,16 +1071,10 @@ bacon_status bacon_compress_host(bacon_ctx* ctx, int requests, const void* q_win
         kos[i] = static_cast<uint16_t*>(ctx->hko_buf) + o_pair * i;
         vos[i] = static_cast<uint16_t*>(ctx->hvo_buf) + o_pair * i;
     }
-    // The TMA descriptors of every request's staging buffers go to the
-    // device first (cached across calls while the buffers stay the same): a
-    // descriptor copy queued on the compute stream after the uploads would
-    // wait behind all of them in the copy engine and hold back the first
-    // request's kernels until the last upload had landed.
-    {
-        rc = upload_maps(ctx, ctx->d_maps, ctx->h_maps, ctx->maps_ev, ctx->map_key, ctx->map_key_N,
-                         kMaxPairs, 0, pairs, qs, ks, seq_len, cs);
-        if (rc != BACON_OK) return rc;
-    }
+    // (The staging buffers are contiguous, so the window kernels take their
+    // TMA descriptors as parameters: a descriptor copy queued on the compute
+    // stream behind the uploads would wait for all of them in the copy
+    // engine.)
     BACON_CUDA(cudaEventRecord(ctx->ev_done[0], cs), "event");  // uploads start after earlier work
     BACON_CUDA(cudaStreamWaitEvent(ctx->h2d, ctx->ev_done[0], 0), "event wait");
     for (int r = 0; r < requests; ++r) {

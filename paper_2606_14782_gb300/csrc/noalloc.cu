@@ -5,8 +5,8 @@
 // must not pay the implicit device-wide synchronisation of cudaMalloc /
 // cudaFree in the middle of prefill.  For them, bacon_window_scores_noalloc
 // runs the same three window kernels as the context-based calls, but keeps
-// their scratch (pass-1 partial statistics, the per-row normalisers and the
-// two TMA descriptors) in one file-scope __device__ array instead of
+// their scratch (pass-1 partial statistics and the per-row normalisers) in
+// one file-scope __device__ array instead of
 // context-owned buffers.
 //
 // The call returns before its kernels run, so a device-side failure (a
@@ -34,16 +34,13 @@ constexpr int kChunk = 1024;          // pass-1 token chunk, as in the context p
 constexpr int kMaxChunks = kMaxSeq / kChunk;
 constexpr int kMaxDevices = 64;
 
-constexpr int kMapBytes = 2 * sizeof(CUtensorMap);  // K map, window-query map
-constexpr int kErrSlots = 2;                        // 16 bytes holding the error word
+constexpr int kErrSlots = 2;          // 16 bytes holding the error word
 
 // [units][chunks][rows] partial (max, sum) pairs, then [units][rows] fp32
-// normalisers packed two per float2, then the two 128-byte TMA descriptors,
-// then the device error word.  About 528 KiB, held by every GPU that loads
-// the library until the process exits.
+// normalisers packed two per float2, then the device error word.  About
+// 528 KiB, held by every GPU that loads the library until the process exits.
 static __device__ __align__(256) float2
-    g_scratch[kMaxTotalRows * kMaxChunks + kMaxTotalRows / 2 + kMapBytes / sizeof(float2) +
-              kErrSlots];
+    g_scratch[kMaxTotalRows * kMaxChunks + kMaxTotalRows / 2 + kErrSlots];
 
 std::mutex g_setup_mutex;
 void* g_scratch_addr[kMaxDevices] = {};
@@ -126,24 +123,18 @@ bacon_status bacon_window_scores_noalloc(int kv_heads, int q_heads, int head_dim
     const int chunks = (seq_len + kChunk - 1) / kChunk;
     float2* partial = scratch;
     float* lse2 = reinterpret_cast<float*>(scratch + (size_t)kMaxTotalRows * kMaxChunks);
-    CUtensorMap* maps =
-        reinterpret_cast<CUtensorMap*>(scratch + (size_t)kMaxTotalRows * kMaxChunks + kMaxTotalRows / 2);
     int* err = reinterpret_cast<int*>(scratch + (size_t)kMaxTotalRows * kMaxChunks +
-                                      kMaxTotalRows / 2 + kMapBytes / sizeof(float2));
-    // descriptors are encoded on the host and copied from this stack buffer;
-    // a copy from pageable memory is staged before cudaMemcpyAsync returns
-    alignas(64) CUtensorMap host_maps[2];
-    if (!encode_rows_map(&host_maps[0], k, head_dim, (long long)kv_heads * seq_len, kTcKBoxRows) ||
-        !encode_rows_map(&host_maps[1], q_win, head_dim, (long long)q_heads * window, kTcQBoxRows))
+                                      kMaxTotalRows / 2);
+    const long long krows = (long long)kv_heads * seq_len, qrows = (long long)q_heads * window;
+    TcArgs a;
+    TcMaps m;  // the TMA descriptors are kernel parameters
+    if (!encode_rows_map(&m.k, k, head_dim, krows, 1, krows * head_dim * 2, kTcKBoxRows) ||
+        !encode_rows_map(&m.q, q_win, head_dim, qrows, 1, qrows * head_dim * 2, kTcQBoxRows))
         return BACON_ECUDA;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    if (cudaMemcpyAsync(maps, host_maps, sizeof host_maps, cudaMemcpyHostToDevice, st) != cudaSuccess)
-        return BACON_ECUDA;
     // the error word must start at zero for this call
     if (cudaMemsetAsync(err, 0, sizeof(int), st) != cudaSuccess) return BACON_ECUDA;
-    TcArgs a;
-    a.kmaps = maps;
-    a.qmaps = maps + 1;
+    a.kmaps = a.qmaps = nullptr;
     a.s = s;
     a.chunks = chunks;
     a.total_chunks = s.units * chunks;
@@ -155,9 +146,9 @@ bacon_status bacon_window_scores_noalloc(int kv_heads, int q_heads, int head_dim
     a.err = err;
     TcArgs a1 = a;
     a1.fault = take_fault();
-    cudaError_t e = launch_window_stats_tc(a1, st);
+    cudaError_t e = launch_window_stats_tc(a1, m, st);
     if (e == cudaSuccess) e = launch_window_combine(s, chunks, partial, lse2, st);
-    if (e == cudaSuccess) e = launch_window_scores_tc(a, st);
+    if (e == cudaSuccess) e = launch_window_scores_tc(a, m, st);
     if (e == cudaSuccess) {
         const size_t n = (size_t)kv_heads * seq_len;
         const size_t blocks = (n + 255) / 256;

@@ -99,7 +99,7 @@ __device__ inline void unit_range(int units, int* u0, int* u1)
 // ---------------------------------------------------------------- producer
 
 template <int D>
-__device__ void produce(const TcArgs& a, const Layout& L, uint8_t* sm, const Bars& b)
+__device__ void produce(const TcArgs& a, const TcMaps& maps, const Layout& L, uint8_t* sm, const Bars& b)
 {
     constexpr int H = D / 64;
     const Shape& s = a.s;
@@ -113,19 +113,22 @@ __device__ void produce(const TcArgs& a, const Layout& L, uint8_t* sm, const Bar
         const uint64_t kpol = tc::l2_evict_first_policy();  // K is read once
         for (int u = u0; u < u1 && ok; ++u, ++n) {
             const int pair = u / s.hkv, h = u - pair * s.hkv;
+            const CUtensorMap* km = a.kmaps ? a.kmaps + pair : &maps.k;
+            const CUtensorMap* qm = a.qmaps ? a.qmaps + pair : &maps.q;
+            const int kz = a.kmaps ? 0 : pair, qz = a.qmaps ? 0 : pair;
             const int slot = n & 1, use = n >> 1;
             if (!tc::mbar_wait(b.q_empty(slot), (use & 1) ^ 1, b.abort())) { ok = false; break; }
             tc::mbar_arrive_expect_tx(b.q_full(slot), L.q_slot);
             for (int kh = 0; kh < H; ++kh)
-                tc::tma_load_2d(sm + L.q + slot * L.q_slot + kh * L.q_half, a.qmaps + pair, kh * 64,
-                                h * s.rows, b.q_full(slot));
+                tc::tma_load_3d(sm + L.q + slot * L.q_slot + kh * L.q_half, qm, kh * 64,
+                                h * s.rows, qz, b.q_full(slot));
             for (int t = 0; t < ntiles; ++t, ++kt) {
                 const int st = kt % kStages, m = kt / kStages;
                 if (!tc::mbar_wait(b.k_empty(st), (m & 1) ^ 1, b.abort())) { ok = false; break; }
                 tc::mbar_arrive_expect_tx(b.k_full(st), L.k_stage);
                 for (int kh = 0; kh < H; ++kh)
-                    tc::tma_load_2d_hint(sm + L.k + st * L.k_stage + kh * kTok * 128, a.kmaps + pair,
-                                         kh * 64, h * s.N + t * kTok, b.k_full(st), kpol);
+                    tc::tma_load_3d_hint(sm + L.k + st * L.k_stage + kh * kTok * 128, km, kh * 64,
+                                         h * s.N + t * kTok, kz, b.k_full(st), kpol);
             }
         }
         if (!ok) raise_abort(b, a.err);
@@ -366,7 +369,7 @@ __device__ void epilogue(const TcArgs& a, const Layout& L, uint8_t* sm, const Ba
 }
 
 template <int D, bool SPEC>
-__global__ void __launch_bounds__(kThreads, 1) window_onepass_kernel(TcArgs a)
+__global__ void __launch_bounds__(kThreads, 1) window_onepass_kernel(TcArgs a, const __grid_constant__ TcMaps maps)
 {
     extern __shared__ uint8_t smem_raw[];
     uint8_t* sm = reinterpret_cast<uint8_t*>(
@@ -391,7 +394,12 @@ __global__ void __launch_bounds__(kThreads, 1) window_onepass_kernel(TcArgs a)
         tc::st_shared_volatile(b.abort(), 0u);
         tc::fence_barrier_init();
     }
+    if (threadIdx.x == 32) {
+        if (!a.kmaps) tc::tma_prefetch_desc(&maps.k);
+        if (!a.qmaps) tc::tma_prefetch_desc(&maps.q);
+    }
     if (warp == 1) {
+        __syncwarp();
         tc::tmem_alloc(b.tmem_slot(), 512);
         tc::tmem_relinquish();
     }
@@ -400,7 +408,7 @@ __global__ void __launch_bounds__(kThreads, 1) window_onepass_kernel(TcArgs a)
     tc::fence_after_sync();
 
     if (warp == 0)
-        produce<D>(a, L, sm, b);
+        produce<D>(a, maps, L, sm, b);
     else if (warp == 1) {
         if (tc::elect_one()) issue<D>(a, L, sm, b);
     } else {
@@ -425,7 +433,7 @@ int num_sms_onepass()
 }
 
 template <int D, bool SPEC>
-cudaError_t launch_d(const TcArgs& a, cudaStream_t st)
+cudaError_t launch_d(const TcArgs& a, const TcMaps& m, cudaStream_t st)
 {
     const Layout L = layout<D>();
     size_t bytes = L.total + 1024;
@@ -435,7 +443,7 @@ cudaError_t launch_d(const TcArgs& a, cudaStream_t st)
     if (e != cudaSuccess) return e;
     const int sms = num_sms_onepass();
     const int grid = a.s.units < sms ? a.s.units : sms;
-    window_onepass_kernel<D, SPEC><<<grid, kThreads, bytes, st>>>(a);
+    window_onepass_kernel<D, SPEC><<<grid, kThreads, bytes, st>>>(a, m);
     return cudaGetLastError();
 }
 
@@ -446,12 +454,12 @@ bool window_onepass_fits(const Shape& s)
     return s.rows <= kRows && (s.d == 64 || s.d == 128) && (s.N + kTok - 1) / kTok <= kMaxTiles;
 }
 
-cudaError_t launch_window_onepass(const TcArgs& a, cudaStream_t st)
+cudaError_t launch_window_onepass(const TcArgs& a, const TcMaps& m, cudaStream_t st)
 {
     if (!window_onepass_fits(a.s)) return cudaErrorInvalidValue;
     const bool spec = a.s.N == 1024 && a.s.W == 32 && a.s.rows == kRows;
-    if (a.s.d == 128) return spec ? launch_d<128, true>(a, st) : launch_d<128, false>(a, st);
-    return spec ? launch_d<64, true>(a, st) : launch_d<64, false>(a, st);
+    if (a.s.d == 128) return spec ? launch_d<128, true>(a, m, st) : launch_d<128, false>(a, m, st);
+    return spec ? launch_d<64, true>(a, m, st) : launch_d<64, false>(a, m, st);
 }
 
 }  // namespace bacon

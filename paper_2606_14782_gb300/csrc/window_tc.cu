@@ -216,7 +216,7 @@ __device__ __forceinline__ void write_bias(const TcArgs& a, uint8_t* bias, int u
 // window rows are reloaded once the previous unit's MMAs have released them
 // (pass 2 also rewrites the bias operand, a second arrival on q_full).
 template <int D, int PASS>
-__device__ __forceinline__ void produce(const TcArgs& a, const Smem& L, uint8_t* sm, const Bars& b,
+__device__ __forceinline__ void produce(const TcArgs& a, const TcMaps& maps, const Smem& L, uint8_t* sm, const Bars& b,
                                         int stages, int q_rows, int q_slots, const JobTable& jt)
 {
     constexpr int H = D / 64;
@@ -238,11 +238,13 @@ __device__ __forceinline__ void produce(const TcArgs& a, const Smem& L, uint8_t*
             if (!ok) break;
             uint8_t* qdst = sm + L.q + slot * L.q_slot;
             if (lane == 0) {
+                const CUtensorMap* qm = a.qmaps ? a.qmaps + pair : &maps.q;
+                const int qz = a.qmaps ? 0 : pair;
                 tc::mbar_arrive_expect_tx(b.q_full(slot), L.q_slot);
                 for (int kh = 0; kh < H; ++kh)
                     for (int rb = 0; rb < q_rows / kQBox; ++rb)
-                        tc::tma_load_2d(qdst + kh * L.q_half + rb * kQBox * 128, a.qmaps + pair,
-                                        kh * 64, h * s.rows + rb * kQBox, b.q_full(slot));
+                        tc::tma_load_3d(qdst + kh * L.q_half + rb * kQBox * 128, qm, kh * 64,
+                                        h * s.rows + rb * kQBox, qz, b.q_full(slot));
             }
             if (PASS == 2) {
                 write_bias(a, sm + L.bias + slot * L.bias_slot, u, jt, inv_c);
@@ -254,6 +256,8 @@ __device__ __forceinline__ void produce(const TcArgs& a, const Smem& L, uint8_t*
             cur_u = u;
         }
         if (lane == 0) {
+            const CUtensorMap* km = a.kmaps ? a.kmaps + pair : &maps.k;
+            const int kz = a.kmaps ? 0 : pair;
             const int t1 = min(ntiles, (ci + 1) * kTilesPerChunk);
             for (int t = ci * kTilesPerChunk; t < t1; ++t, ++kt) {
                 const int st = kt % stages, n = kt / stages;
@@ -263,9 +267,8 @@ __device__ __forceinline__ void produce(const TcArgs& a, const Smem& L, uint8_t*
                 if (PASS == 1 && a.fault == 1 && blockIdx.x == 0 && kt == 0) continue;
                 tc::mbar_arrive_expect_tx(b.k_full(st), L.k_stage);
                 for (int kh = 0; kh < H; ++kh)
-                    tc::tma_load_2d_hint(sm + L.k + st * L.k_stage + kh * kTileTok * 128,
-                                         a.kmaps + pair, kh * 64, h * s.N + t * kTileTok,
-                                         b.k_full(st), kpol);
+                    tc::tma_load_3d_hint(sm + L.k + st * L.k_stage + kh * kTileTok * 128, km,
+                                         kh * 64, h * s.N + t * kTileTok, kz, b.k_full(st), kpol);
             }
         }
         ok = __shfl_sync(0xffffffffu, ok, 0);
@@ -885,7 +888,7 @@ __global__ void lse_from_prefill_kernel(Shape s, LseTable t, float* __restrict__
 // --------------------------------------------------------------- kernels
 
 template <int D, int PASS>
-__global__ void __launch_bounds__(kThreads, 1) window_tc_kernel(TcArgs a, Plan pl)
+__global__ void __launch_bounds__(kThreads, 1) window_tc_kernel(TcArgs a, Plan pl, const __grid_constant__ TcMaps maps)
 {
     extern __shared__ uint8_t smem_raw[];
     uint8_t* sm = reinterpret_cast<uint8_t*>(
@@ -916,7 +919,12 @@ __global__ void __launch_bounds__(kThreads, 1) window_tc_kernel(TcArgs a, Plan p
         tc::st_shared_volatile(b.abort(), 0u);
         tc::fence_barrier_init();
     }
+    if (threadIdx.x == 32) {
+        if (!a.kmaps) tc::tma_prefetch_desc(&maps.k);
+        if (!a.qmaps) tc::tma_prefetch_desc(&maps.q);
+    }
     if (warp == 1) {
+        __syncwarp();
         tc::tmem_alloc(b.tmem_slot(), kTmemCols);
         tc::tmem_relinquish();
     }
@@ -943,7 +951,7 @@ __global__ void __launch_bounds__(kThreads, 1) window_tc_kernel(TcArgs a, Plan p
     tc::fence_after_sync();
 
     if (warp == 0) {
-        produce<D, PASS>(a, L, sm, b, pl.stages, pl.q_rows, pl.q_slots, jt);
+        produce<D, PASS>(a, maps, L, sm, b, pl.stages, pl.q_rows, pl.q_slots, jt);
     } else if (warp == 1) {
         if (tc::elect_one()) {
             const uint32_t ones_stride = pl.ones_atom ? 0u : 1024u;
@@ -1008,7 +1016,7 @@ int num_sms()
 }
 
 template <int D, int PASS>
-cudaError_t launch_impl(const TcArgs& a, cudaStream_t st)
+cudaError_t launch_impl(const TcArgs& a, const TcMaps& m, cudaStream_t st)
 {
     const int rows = a.s.rows;
     const size_t budget = 227 * 1024 - 1024;
@@ -1053,7 +1061,7 @@ cudaError_t launch_impl(const TcArgs& a, cudaStream_t st)
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
     if (e != cudaSuccess) return e;
     const int grid = a.total_chunks < num_sms() ? a.total_chunks : num_sms();
-    window_tc_kernel<D, PASS><<<grid, kThreads, bytes, st>>>(a, pl);
+    window_tc_kernel<D, PASS><<<grid, kThreads, bytes, st>>>(a, pl, m);
     return cudaGetLastError();
 }
 
@@ -1077,17 +1085,17 @@ cudaError_t launch_window_combine(const Shape& s, int chunks, const float2* part
 }
 
 
-cudaError_t launch_window_stats_tc(const TcArgs& a, cudaStream_t st)
+cudaError_t launch_window_stats_tc(const TcArgs& a, const TcMaps& m, cudaStream_t st)
 {
-    if (a.s.d == 128) return launch_impl<128, 1>(a, st);
-    if (a.s.d == 64) return launch_impl<64, 1>(a, st);
+    if (a.s.d == 128) return launch_impl<128, 1>(a, m, st);
+    if (a.s.d == 64) return launch_impl<64, 1>(a, m, st);
     return cudaErrorInvalidValue;
 }
 
-cudaError_t launch_window_scores_tc(const TcArgs& a, cudaStream_t st)
+cudaError_t launch_window_scores_tc(const TcArgs& a, const TcMaps& m, cudaStream_t st)
 {
-    if (a.s.d == 128) return launch_impl<128, 2>(a, st);
-    if (a.s.d == 64) return launch_impl<64, 2>(a, st);
+    if (a.s.d == 128) return launch_impl<128, 2>(a, m, st);
+    if (a.s.d == 64) return launch_impl<64, 2>(a, m, st);
     return cudaErrorInvalidValue;
 }
 
@@ -1101,7 +1109,8 @@ using EncodeFn = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, voi
 EncodeFn g_encode = nullptr;
 }  // namespace
 
-bool encode_rows_map(CUtensorMap* out, const void* base, int d, long long rows, int box_rows)
+bool encode_rows_map(CUtensorMap* out, const void* base, int d, long long rows, int pairs,
+                     long long pair_bytes, int box_rows)
 {
     if (!g_encode) {
         void* fn = nullptr;
@@ -1112,11 +1121,11 @@ bool encode_rows_map(CUtensorMap* out, const void* base, int d, long long rows, 
             return false;
         g_encode = reinterpret_cast<EncodeFn>(fn);
     }
-    cuuint64_t dims[2] = {(cuuint64_t)d, (cuuint64_t)rows};
-    cuuint64_t strides[1] = {(cuuint64_t)d * 2};
-    cuuint32_t box[2] = {64, (cuuint32_t)box_rows};
-    cuuint32_t estr[2] = {1, 1};
-    return g_encode(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides,
+    cuuint64_t dims[3] = {(cuuint64_t)d, (cuuint64_t)rows, (cuuint64_t)pairs};
+    cuuint64_t strides[2] = {(cuuint64_t)d * 2, (cuuint64_t)pair_bytes};
+    cuuint32_t box[3] = {64, (cuuint32_t)box_rows, 1};
+    cuuint32_t estr[3] = {1, 1, 1};
+    return g_encode(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides,
                     box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
                     CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                     CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;

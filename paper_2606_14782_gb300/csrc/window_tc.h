@@ -8,10 +8,26 @@
 
 namespace bacon {
 
+// The TMA descriptors travel as kernel parameters: when the (request, layer)
+// pairs' tensors follow each other at one distance (a contiguous batch, or a
+// single pair) one 3-D map, whose outermost coordinate is the pair, covers
+// them all, and nothing has to be copied to the device before the launch.
+// Per pair it reads exactly what a map of that pair alone reads (rows beyond
+// the pair's own are zero).  A table of one map per pair has to be encoded and
+// copied first, and the next call waits for that copy: without it, 28 layers of a 6528-token prompt
+// scored one by one take 2.35 instead of 2.64 ms.  Pairs at uneven distances
+// take the table of one map each.  (The maps are a parameter of their own:
+// inside TcArgs, whose address would then escape, the window kernels spilled
+// and a 4 x 16384-token step took 1 % longer.)
+struct TcMaps {
+    CUtensorMap k;  // [pairs][Hkv * N][d]
+    CUtensorMap q;  // [pairs][Hq * W][d]
+};
+
 // One launch covers every (request, layer, kv-head) unit of a call.
 struct TcArgs {
-    const CUtensorMap* kmaps;  // [pairs] 2-D maps over each pair's K, [Hkv * N][d]
-    const CUtensorMap* qmaps;  // [pairs] 2-D maps over each pair's window queries, [Hq * W][d]
+    const CUtensorMap* kmaps;  // device table [pairs], each one pair's K, or null (TcMaps)
+    const CUtensorMap* qmaps;  // device table [pairs] of the window queries, or null (TcMaps)
     Shape s;
     int chunks;                // 1024-token chunks per unit
     int total_chunks;          // units * chunks
@@ -31,8 +47,8 @@ constexpr int kTcChunkTokens = 1024;
 int window_tc_max_rows();
 
 // Pass 1 / pass 2 on the tensor cores, and the merge between them.
-cudaError_t launch_window_stats_tc(const TcArgs& a, cudaStream_t st);
-cudaError_t launch_window_scores_tc(const TcArgs& a, cudaStream_t st);
+cudaError_t launch_window_stats_tc(const TcArgs& a, const TcMaps& m, cudaStream_t st);
+cudaError_t launch_window_scores_tc(const TcArgs& a, const TcMaps& m, cudaStream_t st);
 cudaError_t launch_window_combine(const Shape& s, int chunks, const float2* partial, float* lse2,
                                   cudaStream_t st);
 
@@ -40,7 +56,7 @@ cudaError_t launch_window_combine(const Shape& s, int chunks, const float2* part
 // window rows and 1024 tokens): B, Q and E as the two passes give them,
 // without the partial statistics or the merge.
 bool window_onepass_fits(const Shape& s);
-cudaError_t launch_window_onepass(const TcArgs& a, cudaStream_t st);
+cudaError_t launch_window_onepass(const TcArgs& a, const TcMaps& m, cudaStream_t st);
 
 // Per (request, layer) natural-log softmax normalisers of the window rows,
 // [Hq][W] fp32, as a prefill attention kernel produces them.
@@ -50,9 +66,12 @@ struct LseTable {
 cudaError_t launch_lse_from_prefill(const Shape& s, const LseTable& t, float* lse2,
                                     cudaStream_t st);
 
-// 2-D tensor map over `rows` rows of d bf16 values at `base`: boxes of
-// 64 columns x box_rows rows, 128-byte swizzle, zero fill out of bounds.
-bool encode_rows_map(CUtensorMap* out, const void* base, int d, long long rows, int box_rows);
+// Tensor map over `pairs` blocks of `rows` rows of d bf16 values, the first at
+// `base`, `pair_bytes` apart (a multiple of the row's bytes, at least a
+// block's, below 2^40): boxes of 64 columns x box_rows rows of one block,
+// 128-byte swizzle, zero fill out of bounds.
+bool encode_rows_map(CUtensorMap* out, const void* base, int d, long long rows, int pairs,
+                     long long pair_bytes, int box_rows);
 
 // Box heights of the K maps (one 128-token tile) and window-query maps.
 constexpr int kTcKBoxRows = 128;
