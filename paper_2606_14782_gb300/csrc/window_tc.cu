@@ -21,9 +21,11 @@
 //                  a thread owns one token and a share of a job's columns
 //                  (32-column slices, or one 64-column range of a 224-column
 //                  job).
-// Each CTA takes a contiguous range of 1024-token chunks of the flattened
-// (unit, chunk) space, so it reloads the window rows only when its range
-// crosses into the next (request, layer, kv-head).  The epilogue groups meet
+// Each CTA takes a contiguous range of the flattened work, so it reloads the
+// window rows only when its range crosses into the next (request, layer,
+// kv-head): pass 1 of the (unit, 1024-token chunk) space, or of (unit, chunk,
+// 128-row block) when there are too few chunks to fill the GPU; pass 2 of
+// the (unit, 128-token tile) space.  The epilogue groups meet
 // through shared-memory slots and arrival counters, never at a barrier.
 // The epilogues are bound by instruction issue, so the common plans are
 // compiled with their job counts, job sizes and window as constants.
@@ -75,6 +77,8 @@ struct Plan {
     int q_rows, n_jobs, granules, stages, nbuf_log2, bias_rows, ones_atom;
     int q_slots;   // 2: the next unit's window rows load while this unit's MMAs run
     int last_m64;  // pass 1: the last row block holds 64 window rows (an M = 64 job)
+    int blocks;    // pass 1: row blocks of a unit
+    int by_block;  // pass 1: a work item is one row block of a chunk
 };
 
 constexpr uint32_t kOnesBytes = 128u * 128u;
@@ -146,11 +150,52 @@ __device__ inline void raise_abort(const Bars& b, int* err)
     if (err) atomicCAS(err, 0, tc::kErrTimeout);
 }
 
-// Range of global chunks [c0, c1) owned by this CTA.
-__device__ inline void chunk_range(int total, int* c0, int* c1)
+// Range of work items [g0, g1) owned by this CTA.
+__device__ __forceinline__ void item_range(int total, int* g0, int* g1)
 {
-    *c0 = (int)(((long long)blockIdx.x * total) / gridDim.x);
-    *c1 = (int)(((long long)(blockIdx.x + 1) * total) / gridDim.x);
+    *g0 = (int)(((long long)blockIdx.x * total) / gridDim.x);
+    *g1 = (int)(((long long)(blockIdx.x + 1) * total) / gridDim.x);
+}
+
+// A run of tiles [t0, t1) of one unit against its window rows (all of them,
+// or row block rb: `key` tells the loads of window rows apart).
+struct Segment {
+    int u, t0, t1, rb, key;
+};
+
+// The segment that starts at work item g of [g, g1), and the item after it.
+// Pass 1: one chunk (by_block: of one row block).  Pass 2: the unit's tiles
+// up to g1: items are tiles, so that shares differ by one tile (256 units of
+// 24 tiles on 152 CTAs: 41 tiles at most, where whole chunks gave some of
+// them 48).  Pass 2 by chunk and by tile, us per launch: 52.7 and 47.9 at
+// that shape (32 / 8 heads, 2 x 16 layers x 3001 tokens), 80.4 and 72.8 (28
+// layers x 28 / 4 heads x 6528 tokens), 605 and 579 (4 x 28 layers x 16384
+// tokens), 23.4 and 13.9 (one layer x 6528 tokens).
+template <int PASS>
+__device__ __forceinline__ Segment segment_at(const TcArgs& a, const Plan& pl, int ntiles, int g,
+                                              int g1, int* next)
+{
+    Segment s;
+    s.rb = 0;
+    if (PASS == 1) {
+        int c = g;
+        if (pl.by_block) {
+            c = g / pl.blocks;
+            s.rb = g - c * pl.blocks;
+        }
+        s.u = c / a.chunks;
+        s.t0 = (c - s.u * a.chunks) * kTilesPerChunk;
+        s.t1 = min(ntiles, s.t0 + kTilesPerChunk);
+        s.key = pl.by_block ? s.u * pl.blocks + s.rb : s.u;
+        *next = g + 1;
+    } else {
+        s.u = g / ntiles;
+        s.t0 = g - s.u * ntiles;
+        s.t1 = min(ntiles, s.t0 + (g1 - g));
+        s.key = s.u;
+        *next = g + (s.t1 - s.t0);
+    }
+    return s;
 }
 
 // Jobs of one tile: the window rows, in 16-row granules, split into n_jobs
@@ -216,23 +261,25 @@ __device__ __forceinline__ void write_bias(const TcArgs& a, uint8_t* bias, int u
 // window rows are reloaded once the previous unit's MMAs have released them
 // (pass 2 also rewrites the bias operand, a second arrival on q_full).
 template <int D, int PASS>
-__device__ __forceinline__ void produce(const TcArgs& a, const TcMaps& maps, const Smem& L, uint8_t* sm, const Bars& b,
-                                        int stages, int q_rows, int q_slots, const JobTable& jt)
+__device__ __forceinline__ void produce(const TcArgs& a, const TcMaps& maps, const Plan& pl,
+                                        const Smem& L, uint8_t* sm, const Bars& b,
+                                        const JobTable& jt)
 {
+    const int stages = pl.stages, q_slots = pl.q_slots;
     constexpr int H = D / 64;
     const Shape& s = a.s;
     const int lane = threadIdx.x & 31;
     const int ntiles = (s.N + kTileTok - 1) / kTileTok;
     const float inv_c = sqrtf((float)D) / kLog2e;
-    int c0, c1;
-    chunk_range(a.total_chunks, &c0, &c1);
-    int cur_u = -1, qloads = 0, kt = 0;
+    int g0, g1;
+    item_range(a.items, &g0, &g1);
+    int cur = -1, qloads = 0, kt = 0;
     bool ok = true;
     const uint64_t kpol = tc::l2_evict_first_policy();  // K is read once per pass
-    for (int g = c0; g < c1 && ok; ++g) {
-        const int u = g / a.chunks, ci = g - u * a.chunks;
-        const int pair = u / s.hkv, h = u - pair * s.hkv;
-        if (u != cur_u) {
+    for (int g = g0; g < g1 && ok;) {
+        const Segment sg = segment_at<PASS>(a, pl, ntiles, g, g1, &g);
+        const int u = sg.u, pair = u / s.hkv, h = u - pair * s.hkv;
+        if (sg.key != cur) {
             const int slot = qloads % q_slots, use = qloads / q_slots;
             ok = __all_sync(0xffffffffu, tc::mbar_wait(b.q_empty(slot), (use & 1) ^ 1, b.abort()));
             if (!ok) break;
@@ -240,11 +287,16 @@ __device__ __forceinline__ void produce(const TcArgs& a, const TcMaps& maps, con
             if (lane == 0) {
                 const CUtensorMap* qm = a.qmaps ? a.qmaps + pair : &maps.q;
                 const int qz = a.qmaps ? 0 : pair;
-                tc::mbar_arrive_expect_tx(b.q_full(slot), L.q_slot);
+                // the segment's window rows, in 64-row boxes from row r0 (a
+                // last block of 64 rows fills half of the slot)
+                const int r0 = 128 * sg.rb;
+                const int boxes = (pl.last_m64 && pl.by_block && sg.rb == pl.blocks - 1)
+                                      ? 1 : pl.q_rows / kQBox;
+                tc::mbar_arrive_expect_tx(b.q_full(slot), (uint32_t)(H * boxes * kQBox) * 128u);
                 for (int kh = 0; kh < H; ++kh)
-                    for (int rb = 0; rb < q_rows / kQBox; ++rb)
-                        tc::tma_load_3d(qdst + kh * L.q_half + rb * kQBox * 128, qm, kh * 64,
-                                        h * s.rows + rb * kQBox, qz, b.q_full(slot));
+                    for (int i = 0; i < boxes; ++i)
+                        tc::tma_load_3d(qdst + kh * L.q_half + i * kQBox * 128, qm, kh * 64,
+                                        h * s.rows + r0 + i * kQBox, qz, b.q_full(slot));
             }
             if (PASS == 2) {
                 write_bias(a, sm + L.bias + slot * L.bias_slot, u, jt, inv_c);
@@ -253,13 +305,12 @@ __device__ __forceinline__ void produce(const TcArgs& a, const TcMaps& maps, con
                 if (lane == 0) tc::mbar_arrive(b.q_full(slot));
             }
             ++qloads;
-            cur_u = u;
+            cur = sg.key;
         }
         if (lane == 0) {
             const CUtensorMap* km = a.kmaps ? a.kmaps + pair : &maps.k;
             const int kz = a.kmaps ? 0 : pair;
-            const int t1 = min(ntiles, (ci + 1) * kTilesPerChunk);
-            for (int t = ci * kTilesPerChunk; t < t1; ++t, ++kt) {
+            for (int t = sg.t0; t < sg.t1; ++t, ++kt) {
                 const int st = kt % stages, n = kt / stages;
                 if (!tc::mbar_wait(b.k_empty(st), (n & 1) ^ 1, b.abort())) { ok = false; break; }
                 // injected fault (tests only): the first load never arrives, so
@@ -292,32 +343,33 @@ __device__ __forceinline__ void produce(const TcArgs& a, const TcMaps& maps, con
 // Pass 1: A = window rows (M = 128 per row block), B = K tile (N = 128).
 // Pass 2: A = K tile (M = 128 tokens), B = window rows (N = n_h per half).
 template <int D, int PASS, int NBUF_LOG2>
-__device__ __forceinline__ void issue(const TcArgs& a, const Smem& L, uint8_t* sm, const Bars& b, int stages,
-                      int q_slots, const JobTable& jt, uint32_t ones_stride, int last_m64)
+__device__ __forceinline__ void issue(const TcArgs& a, const Plan& pl, const Smem& L, uint8_t* sm,
+                                      const Bars& b, const JobTable& jt)
 {
+    const int stages = pl.stages, q_slots = pl.q_slots, last_m64 = pl.last_m64;
+    const uint32_t ones_stride = pl.ones_atom ? 0u : 1024u;
     const Shape& s = a.s;
     const int ntiles = (s.N + kTileTok - 1) / kTileTok;
     const uint32_t tmem = tc::ld_shared(b.tmem_slot());
     const uint32_t sbase = smem_u32(sm);
     constexpr int buf_mask = (1 << NBUF_LOG2) - 1;
     constexpr uint32_t buf_cols = (uint32_t)kTmemCols >> NBUF_LOG2;
-    int c0, c1;
-    chunk_range(a.total_chunks, &c0, &c1);
-    int cur_u = -1, cur_slot = 0, qwaits = 0, kt = 0, job = 0;
+    int g0, g1;
+    item_range(a.items, &g0, &g1);
+    int cur = -1, cur_slot = 0, qwaits = 0, kt = 0, job = 0;
     bool ok = true;
-    for (int g = c0; g < c1 && ok; ++g) {
-        const int u = g / a.chunks, ci = g - u * a.chunks;
-        if (u != cur_u) {
-            if (cur_u >= 0) tc::umma_commit(b.q_empty(cur_slot));  // previous unit's MMAs release its slot
+    for (int g = g0; g < g1 && ok;) {
+        const Segment sg = segment_at<PASS>(a, pl, ntiles, g, g1, &g);
+        if (sg.key != cur) {
+            if (cur >= 0) tc::umma_commit(b.q_empty(cur_slot));  // previous unit's MMAs release its slot
             const int slot = qwaits % q_slots, use = qwaits / q_slots;
             if (!tc::mbar_wait(b.q_full(slot), use & 1, b.abort())) { ok = false; break; }
             tc::fence_after_sync();
             ++qwaits;
-            cur_u = u;
+            cur = sg.key;
             cur_slot = slot;
         }
-        const int t1 = min(ntiles, (ci + 1) * kTilesPerChunk);
-        for (int t = ci * kTilesPerChunk; t < t1 && ok; ++t, ++kt) {
+        for (int t = sg.t0; t < sg.t1 && ok; ++t, ++kt) {
             const int st = kt % stages, n = kt / stages;
             if (!tc::mbar_wait(b.k_full(st), n & 1, b.abort())) { ok = false; break; }
             tc::fence_after_sync();
@@ -332,7 +384,7 @@ __device__ __forceinline__ void issue(const TcArgs& a, const Smem& L, uint8_t* s
                 const uint32_t d_tmem = tmem + buf * buf_cols;
                 // pass 1's last row block of 64 window rows: an M = 64 job,
                 // which fills the first 16 lanes of each TMEM lane quarter
-                const int m_rows = (PASS == 1 && last_m64 && j == jt.n_jobs - 1) ? 64 : 128;
+                const int m_rows = (PASS == 1 && last_m64 && sg.rb + j == pl.blocks - 1) ? 64 : 128;
                 const uint32_t idesc = tc::idesc_bf16(m_rows, jt.n(j));
                 const uint32_t qaddr = sbase + L.q + cur_slot * L.q_slot + jt.row0(j) * 128;
                 if (PASS == 2)  // D = -lse2 / c per row (columns of D), then += K Q^T
@@ -410,6 +462,23 @@ __device__ __forceinline__ void row_stats(const float* v, float mx, float c, uns
     m_run = m_new;
 }
 
+// The statistics of one row over the four groups' tokens, in group order.
+__device__ __forceinline__ float2 merge_groups(const float2* mz)
+{
+    float M = -INFINITY;
+#pragma unroll
+    for (int gg = 0; gg < kGroups; ++gg) M = fmaxf(M, mz[gg].x);
+    float Z = 0.f;
+    if (M != -INFINITY) {
+#pragma unroll
+        for (int gg = 0; gg < kGroups; ++gg) {
+            const float zz = mz[gg].y * fast_exp2(mz[gg].x - M);
+            Z = gg == 0 ? zz : Z + zz;
+        }
+    }
+    return make_float2(M, Z);
+}
+
 // Thread = one window row (TMEM lane) x one 32-token quarter (its group) of
 // every job; running (max, sum of 2^x) per row block, merged across the
 // groups at the end of each chunk.  With last_m64 the last row block is an
@@ -440,7 +509,7 @@ __device__ __forceinline__ void epilogue_stats(const TcArgs& a, const Smem& L, u
     const float c = kLog2e * rsqrtf((float)D);
     const unsigned long long c2 = tc::pack2(c, c);
     int c0, c1;
-    chunk_range(a.total_chunks, &c0, &c1);
+    item_range(a.items, &c0, &c1);
     int job = 0, nch = 0, tcount = 0;
     bool ok = true;
     // the last position each of this thread's rows sees (rows of every block)
@@ -564,21 +633,104 @@ __device__ __forceinline__ void epilogue_stats(const TcArgs& a, const Smem& L, u
                 for (int gg = 0; gg < kGroups; ++gg)
                     mz[gg] = gg == group ? (h ? make_float2(m_h, z_h) : make_float2(m_run[rb], z_run[rb]))
                                          : vx[(gg * 4 + rb) * 128];
-                float M = -INFINITY;
-#pragma unroll
-                for (int gg = 0; gg < kGroups; ++gg) M = fmaxf(M, mz[gg].x);
-                float Z = 0.f;
-                if (M != -INFINITY) {
-#pragma unroll
-                    for (int gg = 0; gg < kGroups; ++gg) {
-                        const float zz = mz[gg].y * fast_exp2(mz[gg].x - M);
-                        Z = gg == 0 ? zz : Z + zz;
-                    }
-                }
                 const int r = h ? row_h : rb * 128 + quarter * 32 + lane;
                 if ((!h || (lane & 2) == 0) && r < s.rows)
-                    a.partial[((size_t)u * a.chunks + ci) * s.rows + r] = make_float2(M, Z);
+                    a.partial[((size_t)u * a.chunks + ci) * s.rows + r] = merge_groups(mz);
             }
+            __syncwarp();
+            if (lane == 0) tc::mbar_arrive(b.x_empty(0, quarter));
+        }
+    }
+    if (!ok) raise_abort(b, a.err);
+}
+
+// epilogue_stats for work items of one row block (by_block): the same jobs,
+// the same sums and the same merge of that block's rows, so the partials are
+// the same bits; one job per tile.  A call of few chunks (one layer of 4
+// kv-heads x 6528 tokens: 28) leaves most SMs idle when a chunk is the
+// smallest item; its K tiles are read once per row block instead, from L2.
+__device__ __forceinline__ void epilogue_stats_block(const TcArgs& a, const Plan& pl, const Smem& L,
+                                                     uint8_t* sm, const Bars& b, float c)
+{
+    const Shape& s = a.s;
+    const int ntiles = (s.N + kTileTok - 1) / kTileTok;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int quarter = warp & 3;
+    const int group = (warp - 2) >> 2;
+    const uint32_t tmem = tc::ld_shared(b.tmem_slot()) + ((uint32_t)(quarter * 32) << 16) + group * 32;
+    float2* xchg = reinterpret_cast<float2*>(sm + L.xchg) + quarter * 32 + lane;  // [group][128]
+    const int odd = (lane >> 1) & 1;
+    const unsigned long long c2 = tc::pack2(c, c);
+    int g0, g1;
+    item_range(a.items, &g0, &g1);
+    int job = 0, nitem = 0;
+    bool ok = true;
+    for (int g = g0; g < g1 && ok;) {
+        const Segment sg = segment_at<1>(a, pl, ntiles, g, g1, &g);
+        const bool half = pl.last_m64 && sg.rb == pl.blocks - 1;
+        const int row = sg.rb * 128 + (half ? quarter * 16 + (lane >> 2) + 8 * (lane & 1)
+                                            : quarter * 32 + lane);
+        const int vis = s.N - s.W + row % s.W;  // the last position the row sees
+        float m_run = -INFINITY, z_run = 0.f;
+        for (int t = sg.t0; t < sg.t1; ++t, ++job) {
+            const int tok0 = t * kTileTok + group * 32;
+            const bool need_mask = tok0 + 31 > s.N - s.W;
+            const int buf = job & 3, nb = job >> 2;
+            if (!tc::mbar_wait(b.t_full(buf), nb & 1, b.abort())) { ok = false; break; }
+            tc::fence_after_sync();
+            float v[32], mx;
+            if (half) {
+                tc::tmem_ld16x64b_x16(tmem + buf * 128, v);
+                tc::tmem_ld_wait_regs16(v);
+            } else {
+                tc::tmem_ld32_max(tmem + buf * 128, v, mx);
+                tc::tmem_ld_wait_regs32_max(v, mx);
+            }
+            tc::fence_before_sync();
+            __syncwarp();
+            if (lane == 0) tc::mbar_arrive(b.t_empty(buf));
+            if (half) {
+                if (need_mask) {
+#pragma unroll
+                    for (int j = 0; j < 16; ++j)
+                        if (tok0 + 2 * j + odd > vis) v[j] = -INFINITY;
+                }
+                row_stats<16>(v, max_tree<16>(v), c, c2, m_run, z_run);
+            } else if (need_mask) {
+#pragma unroll
+                for (int j = 0; j < 32; ++j)
+                    if (tok0 + j > vis) v[j] = -INFINITY;
+                row_stats<32, true>(v, max_tree<32>(v), c, c2, m_run, z_run);
+            } else {
+                row_stats<32, false>(v, mx, c, c2, m_run, z_run);
+            }
+        }
+        if (!ok) break;
+        if (half) {
+            const float mo = __shfl_xor_sync(0xffffffffu, m_run, 2);
+            const float zo = __shfl_xor_sync(0xffffffffu, z_run, 2);
+            const float M = fmaxf(m_run, mo);
+            if (M != -INFINITY) z_run = z_run * fast_exp2(m_run - M) + zo * fast_exp2(mo - M);
+            m_run = M;
+        }
+        // the hand-off of epilogue_stats, one row block at a time
+        const int merger = nitem & 3;
+        const uint32_t ph = (uint32_t)nitem & 1u;
+        ++nitem;
+        if (!tc::mbar_wait(b.x_empty(0, quarter), ph ^ 1u, b.abort())) { ok = false; break; }
+        if (group != merger) {
+            xchg[group * 128] = make_float2(m_run, z_run);
+            __syncwarp();
+            if (lane == 0) tc::mbar_arrive(b.x_full(0, quarter));
+        } else {
+            if (!tc::mbar_wait(b.x_full(0, quarter), ph, b.abort())) { ok = false; break; }
+            float2 mz[kGroups];
+#pragma unroll
+            for (int gg = 0; gg < kGroups; ++gg)
+                mz[gg] = gg == group ? make_float2(m_run, z_run) : xchg[gg * 128];
+            if ((!half || (lane & 2) == 0) && row < s.rows)
+                a.partial[((size_t)sg.u * a.chunks + sg.t0 / kTilesPerChunk) * s.rows + row] =
+                    merge_groups(mz);
             __syncwarp();
             if (lane == 0) tc::mbar_arrive(b.x_empty(0, quarter));
         }
@@ -762,8 +914,8 @@ __device__ __forceinline__ bool score_tile(const JobTable& jt, int& job, int jt0
 }
 
 template <int D, bool FASTQ, int NBUF_LOG2, int J, int NPJ, int WQ = 0>
-__device__ __forceinline__ void epilogue_scores(const TcArgs& a, const Smem& L, uint8_t* sm,
-                                                const Bars& b, const JobTable& jt)
+__device__ __forceinline__ void epilogue_scores(const TcArgs& a, const Plan& pl, const Smem& L,
+                                                uint8_t* sm, const Bars& b, const JobTable& jt)
 {
     const Shape& s = a.s;
     const int ntiles = (s.N + kTileTok - 1) / kTileTok;
@@ -780,14 +932,14 @@ __device__ __forceinline__ void epilogue_scores(const TcArgs& a, const Smem& L, 
     k.qmask = 0u;
     for (int g = 0; g < 32; ++g)
         if (16 * g + 15 < s.rows && (16 * g + 15) % s.W == s.W - 1) k.qmask |= 1u << g;
-    int c0, c1;
-    chunk_range(a.total_chunks, &c0, &c1);
+    int g0, g1;
+    item_range(a.items, &g0, &g1);
     int job = 0, ntile = 0;
     bool ok = true;
-    for (int g = c0; g < c1 && ok; ++g) {
-        const int u = g / a.chunks, ci = g - u * a.chunks;
-        const int t1 = min(ntiles, (ci + 1) * kTilesPerChunk);
-        for (int t = ci * kTilesPerChunk; t < t1 && ok; ++t) {
+    for (int g = g0; g < g1 && ok;) {
+        const Segment sg = segment_at<2>(a, pl, ntiles, g, g1, &g);
+        const int u = sg.u;
+        for (int t = sg.t0; t < sg.t1 && ok; ++t) {
             const int tok = t * kTileTok + quarter * 32 + lane;
             const bool need_mask = t * kTileTok + kTileTok - 1 > s.N - s.W;
             unsigned long long bacc[2] = {0ull, 0ull};
@@ -951,20 +1103,21 @@ __global__ void __launch_bounds__(kThreads, 1) window_tc_kernel(TcArgs a, Plan p
     tc::fence_after_sync();
 
     if (warp == 0) {
-        produce<D, PASS>(a, maps, L, sm, b, pl.stages, pl.q_rows, pl.q_slots, jt);
+        produce<D, PASS>(a, maps, pl, L, sm, b, jt);
     } else if (warp == 1) {
         if (tc::elect_one()) {
-            const uint32_t ones_stride = pl.ones_atom ? 0u : 1024u;
             if (pl.nbuf_log2 == 1)
-                issue<D, PASS, 1>(a, L, sm, b, pl.stages, pl.q_slots, jt, ones_stride, pl.last_m64);
+                issue<D, PASS, 1>(a, pl, L, sm, b, jt);
             else
-                issue<D, PASS, 2>(a, L, sm, b, pl.stages, pl.q_slots, jt, ones_stride, pl.last_m64);
+                issue<D, PASS, 2>(a, pl, L, sm, b, jt);
         }
     } else {
         if (PASS == 1)
         {
-            const int nrb = (pl.q_rows + 127) / 128;
-            if (nrb == 4 && pl.last_m64)
+            const int nrb = pl.blocks;
+            if (pl.by_block)
+                epilogue_stats_block(a, pl, L, sm, b, kLog2e * rsqrtf((float)D));
+            else if (nrb == 4 && pl.last_m64)
                 epilogue_stats<D, 4, true>(a, L, sm, b, pl.q_rows, pl.last_m64);
             else if (nrb == 2 && !pl.last_m64)
                 epilogue_stats<D, 2, false>(a, L, sm, b, pl.q_rows, pl.last_m64);
@@ -973,23 +1126,23 @@ __global__ void __launch_bounds__(kThreads, 1) window_tc_kernel(TcArgs a, Plan p
         }
         else if (a.s.W % 16 == 0 && pl.nbuf_log2 == 1) {
             if (pl.n_jobs == 2 && pl.granules == 28 && a.s.W == 64)
-                epilogue_scores<D, true, 1, 2, 14, 64>(a, L, sm, b, jt);
+                epilogue_scores<D, true, 1, 2, 14, 64>(a, pl, L, sm, b, jt);
             else if (pl.n_jobs == 2 && pl.granules == 28)
-                epilogue_scores<D, true, 1, 2, 14>(a, L, sm, b, jt);
+                epilogue_scores<D, true, 1, 2, 14>(a, pl, L, sm, b, jt);
             else if (pl.n_jobs == 2)
-                epilogue_scores<D, true, 1, 2, 0>(a, L, sm, b, jt);
+                epilogue_scores<D, true, 1, 2, 0>(a, pl, L, sm, b, jt);
             else if (pl.n_jobs == 1 && pl.granules == 14 && a.s.W == 32)
-                epilogue_scores<D, true, 1, 1, 14, 32>(a, L, sm, b, jt);
+                epilogue_scores<D, true, 1, 1, 14, 32>(a, pl, L, sm, b, jt);
             else if (pl.n_jobs == 1 && pl.granules == 14)
-                epilogue_scores<D, true, 1, 1, 14>(a, L, sm, b, jt);
+                epilogue_scores<D, true, 1, 1, 14>(a, pl, L, sm, b, jt);
             else if (pl.n_jobs == 1)
-                epilogue_scores<D, true, 1, 1, 0>(a, L, sm, b, jt);
+                epilogue_scores<D, true, 1, 1, 0>(a, pl, L, sm, b, jt);
             else
-                epilogue_scores<D, true, 1, 0, 0>(a, L, sm, b, jt);
+                epilogue_scores<D, true, 1, 0, 0>(a, pl, L, sm, b, jt);
         } else if (a.s.W % 16 == 0)
-            epilogue_scores<D, true, 2, 0, 0>(a, L, sm, b, jt);
+            epilogue_scores<D, true, 2, 0, 0>(a, pl, L, sm, b, jt);
         else  // W % 16 != 0: always four accumulators (see launch_impl)
-            epilogue_scores<D, false, 2, 0, 0>(a, L, sm, b, jt);
+            epilogue_scores<D, false, 2, 0, 0>(a, pl, L, sm, b, jt);
     }
 
     tc::fence_before_sync();
@@ -1015,10 +1168,25 @@ int num_sms()
     return cache[dev];
 }
 
-template <int D, int PASS>
-cudaError_t launch_impl(const TcArgs& a, const TcMaps& m, cudaStream_t st)
+// Pass 1 by row block of a chunk (four times the work items at 448 window
+// rows) instead of by chunk: when it shortens the largest share of a CTA,
+// counted in tiles x row blocks.  A row block alone needs its K tile from L2
+// for one job instead of `blocks` of them, which the factor allows for.  One
+// layer of 4 kv-heads, 448 rows, by chunk and by row block: 18.3 and 10.6 us
+// (6528 tokens: 28 chunks), 18.6 and 16.1 us (16384 tokens: 64 chunks, the
+// largest share 2 items of 8 tiles instead of 1 of 28 tile jobs).
+bool stats_by_block(int chunks, int blocks, int sms)
 {
-    const int rows = a.s.rows;
+    if (blocks == 1) return false;
+    const long long whole = (long long)((chunks + sms - 1) / sms) * blocks;
+    const long long split = ((long long)chunks * blocks + sms - 1) / sms;
+    return 3 * split <= 2 * whole;
+}
+
+template <int D, int PASS>
+cudaError_t launch_impl(const TcArgs& args, const TcMaps& m, cudaStream_t st)
+{
+    const int rows = args.s.rows;
     const size_t budget = 227 * 1024 - 1024;
     // window rows in shared memory: whole 64-row TMA boxes.  Pass 1 runs
     // whole 128-row MMA blocks over them in four 128-column accumulators; the
@@ -1029,13 +1197,24 @@ cudaError_t launch_impl(const TcArgs& a, const TcMaps& m, cudaStream_t st)
     Plan pl;
     pl.q_rows = (rows + kQBox - 1) / kQBox * kQBox;
     pl.last_m64 = (PASS == 1 && pl.q_rows % 128 == 64) ? 1 : 0;
+    pl.blocks = (pl.q_rows + 127) / 128;
     const int granules = (rows + 15) / 16;
+    const int sms = num_sms();
+    TcArgs a = args;
+    if (PASS == 1) {
+        pl.by_block = stats_by_block(a.total_chunks, pl.blocks, sms) ? 1 : 0;
+        a.items = pl.by_block ? a.total_chunks * pl.blocks : a.total_chunks;
+        if (pl.by_block) pl.q_rows = 128;
+    } else {
+        pl.by_block = 0;
+        a.items = a.s.units * ((a.s.N + kTileTok - 1) / kTileTok);
+    }
     Smem L;
     bool fits = false;
     // (a window that is not a multiple of 16 rows always takes 128-row jobs)
     for (int attempt = a.s.W % 16 == 0 ? 0 : 1; attempt < 2 && !fits; ++attempt) {
         const int per_job = PASS == 1 ? 8 : (attempt == 0 ? 16 : 8);  // granules
-        pl.n_jobs = PASS == 1 ? (pl.q_rows + 127) / 128 : (granules + per_job - 1) / per_job;
+        pl.n_jobs = PASS == 1 ? (pl.by_block ? 1 : pl.blocks) : (granules + per_job - 1) / per_job;
         pl.granules = PASS == 1 ? 8 * pl.n_jobs : granules;
         pl.nbuf_log2 = per_job == 16 ? 1 : 2;
         pl.bias_rows = PASS == 2 ? 16 * ((pl.granules + pl.n_jobs - 1) / pl.n_jobs) : 0;
@@ -1060,7 +1239,7 @@ cudaError_t launch_impl(const TcArgs& a, const TcMaps& m, cudaStream_t st)
     cudaError_t e = cudaFuncSetAttribute(window_tc_kernel<D, PASS>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
     if (e != cudaSuccess) return e;
-    const int grid = a.total_chunks < num_sms() ? a.total_chunks : num_sms();
+    const int grid = a.items < sms ? a.items : sms;
     window_tc_kernel<D, PASS><<<grid, kThreads, bytes, st>>>(a, pl, m);
     return cudaGetLastError();
 }

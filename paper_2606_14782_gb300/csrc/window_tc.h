@@ -31,6 +31,7 @@ struct TcArgs {
     Shape s;
     int chunks;                // 1024-token chunks per unit
     int total_chunks;          // units * chunks
+    int items;                 // work items of the launch (set by it)
     float2* partial;           // pass 1 output [units][chunks][rows]
     const float* lse2;         // pass 2 input  [units][rows]
     float* B;                  // pass 2 outputs [units][N]

@@ -1,0 +1,61 @@
+"""The window passes cut their work by the size of the call: pass 1 by chunk
+of a unit or, when that leaves SMs idle, by row block of a chunk, pass 2 by
+tile.  A call of many units and a call of one layer therefore take different
+routes over the same tensors; their final scores must be the same bits."""
+
+import pytest
+import torch
+
+from paper_2606_14782_gb300 import bacon, build, workloads
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _lib():
+    build.build()
+    bacon.load()
+
+
+# window rows G W: one to four row blocks, whole and half last ones, and rows
+# that do not fill their 64-row box
+@pytest.mark.parametrize("group,window,head_dim,seq_len", [
+    (1, 64, 128, 1153),    # 64 rows: one block
+    (4, 34, 64, 1025),     # 136: a half last block of 8 rows
+    (3, 64, 128, 2047),    # 192
+    (4, 64, 64, 1300),     # 256
+    (5, 64, 128, 1100),    # 320
+    (6, 64, 128, 1281),    # 384
+    (7, 64, 64, 1537),     # 448
+    (7, 63, 128, 1111),    # 441: a window that is not a multiple of 16
+    (8, 64, 128, 1024),    # 512
+])
+def test_few_units_and_many_give_the_same_bits(group, window, head_dim, seq_len):
+    layers, requests, hkv = 20, 4, 2  # at least 320 chunks: by chunk
+    wl = workloads.CONFIGS["tiny"].with_(
+        layers=layers, requests=requests, q_heads=group * hkv, kv_heads=hkv, head_dim=head_dim,
+        seq_len=seq_len, window=window, visual=(16, seq_len - 200))
+    x = workloads.generate(wl, seed=9, device="cuda")
+    budget = window + 40
+    ctx = bacon.Context(layers, hkv, group * hkv, head_dim, window, 7, budget,
+                        max_seq_len=seq_len, max_requests=requests, keep_scores=1)
+    _, _, idx = ctx.compress_all_layers(x.qwin, x.k, x.v, budget)
+    whole = {n: ctx.scores(n).view(requests, layers, hkv, seq_len) for n in ("S", "B", "Q")}
+    ctx.sync()
+    st = bacon.State(ctx)
+    for r in (0, requests - 1):
+        st.reset()
+        for l in range(3):
+            S = st.score_layer(l, x.qwin[r, l], x.k[r, l], scores_out=True)
+            assert torch.equal(S, whole["S"][r, l]), (r, l)
+            assert torch.equal(st.select(budget, seq_len), idx[r, l]), (r, l)
+    # the same two passes without a context
+    B, Q, E = (torch.empty(hkv, seq_len, device="cuda") for _ in range(3))
+    rc = bacon.load().bacon_window_scores_noalloc(
+        hkv, group * hkv, head_dim, window, x.qwin[1, 2].data_ptr(), x.k[1, 2].data_ptr(), seq_len,
+        B.data_ptr(), Q.data_ptr(), E.data_ptr(), torch.cuda.current_stream().cuda_stream)
+    assert rc == bacon.BACON_OK
+    ctx.sync()
+    assert torch.equal(B, whole["B"][1, 2]) and torch.equal(Q, whole["Q"][1, 2])
+    st.close()
+    ctx.close()
