@@ -10,6 +10,7 @@ from __future__ import annotations
 
 import ctypes
 import os
+from array import array
 
 import torch
 
@@ -139,8 +140,8 @@ def default_params(**overrides) -> Params:
 
 
 def _stream_ptr(stream) -> int:
-    if stream is None:
-        stream = torch.cuda.current_stream()
+    if stream is None:  # the current stream, without building a Stream object
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
     return stream.cuda_stream
 
 
@@ -160,8 +161,12 @@ def _pair_table(t, pairs):
     [R, layers, ...] tensor."""
     if not t.is_contiguous():
         raise ValueError("tensors must be contiguous")
-    base, stride = t.data_ptr(), t[0, 0].numel() * t.element_size()
-    return _ptr_array([base + stride * i for i in range(pairs)])
+    base = t.data_ptr()
+    stride = t.numel() // (t.shape[0] * t.shape[1]) * t.element_size()
+    # one buffer of addresses instead of one ctypes store per pair: 28 pairs
+    # take 1.5 us instead of 8
+    ptrs = array("Q", range(base, base + stride * pairs, stride) if stride else [base] * pairs)
+    return (_vp * pairs).from_buffer(ptrs)
 
 
 class Context:
@@ -214,9 +219,8 @@ class Context:
             v_out = torch.empty(shape_o, dtype=v.dtype, device=v.device)
         if idx_out is None:
             idx_out = torch.empty(shape_o[:-1], dtype=torch.int32, device=k.device)
-        for t in (qwin, k, v, k_out, v_out, idx_out):
-            if not t.is_contiguous():
-                raise ValueError("tensors must be contiguous")
+        if not idx_out.is_contiguous():
+            raise ValueError("tensors must be contiguous")
         tq, tk, tv, tko, tvo = (_pair_table(t, R * Ly) for t in (qwin, k, v, k_out, v_out))
         _check(load().bacon_compress_all_layers(self.handle, R, tq, tk, tv, N, budget, tko, tvo,
                                                 idx_out.data_ptr(), _stream_ptr(stream)))
@@ -236,9 +240,8 @@ class Context:
         ix = [[torch.empty((self.kv_heads, kept[l]), dtype=torch.int32, device=k.device)
                for l in range(Ly)] for _ in range(R)]
         pairs = [(r, l) for r in range(R) for l in range(Ly)]
-        tq = _ptr_array([qwin[r, l].data_ptr() for r, l in pairs])
-        tk = _ptr_array([k[r, l].data_ptr() for r, l in pairs])
-        tv = _ptr_array([v[r, l].data_ptr() for r, l in pairs])
+        tq, tk, tv = (_pair_table(t, len(pairs)) if t.is_contiguous() else
+                      _ptr_array([t[r, l].data_ptr() for r, l in pairs]) for t in (qwin, k, v))
         tko = _ptr_array([ko[r][l].data_ptr() for r, l in pairs])
         tvo = _ptr_array([vo[r][l].data_ptr() for r, l in pairs])
         tix = _ptr_array([ix[r][l].data_ptr() for r, l in pairs])
