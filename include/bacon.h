@@ -313,7 +313,7 @@ bacon_status bacon_profile_read(bacon_ctx* ctx, double* ms, int* launches, int n
  * code that must not pay the device-wide synchronisation of cudaMalloc /
  * cudaFree in the middle of prefill.  It needs no context: the kernels'
  * scratch (the softmax statistics) lives in one static __device__ array of
- * about 528 KiB, which every GPU that loads the library holds until the
+ * about 512 KiB, which every GPU that loads the library holds until the
  * process exits.
  *
  * Inputs as in the layouts above (q_win [Hq][W][d], k [Hkv][N][d] bf16);
@@ -334,8 +334,8 @@ bacon_status bacon_profile_read(bacon_ctx* ctx, double* ms, int* launches, int n
  * calls whose work can overlap on the GPU (different streams, or several
  * host threads) race and must be serialised by the caller.  The array keeps
  * the last call's contents; its error word, the one entry that must start
- * at zero, is cleared by each call on its stream, and every other entry a
- * call reads it has written first. */
+ * at zero, is cleared again on the stream by the call that set it, and every
+ * other entry a call reads it has written first. */
 bacon_status bacon_window_scores_noalloc(int kv_heads, int q_heads, int head_dim, int window,
                                          const void* q_win, const void* k, int seq_len,
                                          float* B_out, float* Q_out, float* E_out,

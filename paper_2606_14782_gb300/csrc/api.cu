@@ -134,7 +134,6 @@ struct bacon_state {
     float* Q = nullptr;
     float* S = nullptr;
     float* lam = nullptr;
-    float* lse2 = nullptr;
     float2* partial = nullptr;
 };
 
@@ -709,7 +708,6 @@ bacon_status bacon_state_create(bacon_ctx* ctx, bacon_state** out)
     if (e == cudaSuccess) e = dalloc(&st->Q, tok);
     if (e == cudaSuccess) e = dalloc(&st->S, tok);
     if (e == cudaSuccess) e = dalloc(&st->lam, ctx->hkv);
-    if (e == cudaSuccess) e = dalloc(&st->lse2, (size_t)ctx->hkv * ctx->rows);
     if (e == cudaSuccess) e = dalloc(&st->partial, (size_t)ctx->hkv * chunks * ctx->rows);
     if (e != cudaSuccess) {
         cudaGetLastError();
@@ -732,7 +730,7 @@ bacon_status bacon_state_reset(bacon_state* st)
 void bacon_state_destroy(bacon_state* st)
 {
     if (!st) return;
-    void* bufs[] = {st->Ering, st->B, st->Q, st->S, st->lam, st->lse2, st->partial};
+    void* bufs[] = {st->Ering, st->B, st->Q, st->S, st->lam, st->partial};
     for (void* b : bufs)
         if (b) cudaFree(b);
     delete st;
@@ -758,12 +756,12 @@ bacon_status bacon_score_layer(bacon_ctx* ctx, bacon_state* st, int layer, const
 
     const Shape s = shape_of(ctx, 1, 1, seq_len);
     float* Eslot = st->Ering + (size_t)(layer % st->ring) * ctx->hkv * seq_len;
-    TcArgs ta = tc_args(s, st->partial, st->lse2, st->B, st->Q, Eslot, ctx->err);
+    TcArgs ta = tc_args(s, st->partial, nullptr, st->B, st->Q, Eslot, ctx->err);
     TcMaps tm;
     if (!bind_maps(ctx, tm, 1, &q_win, &k, seq_len))
         return fail(BACON_ECUDA, "cuTensorMapEncodeTiled failed");
+    // one layer: pass 2 forms the row normalisers itself
     BACON_CUDA(launch_window_stats_tc(ta, tm, cs), "window_stats launch");
-    BACON_CUDA(launch_window_combine(s, ta.chunks, st->partial, st->lse2, cs), "window_combine launch");
     BACON_CUDA(launch_window_scores_tc(ta, tm, cs), "window_scores launch");
 
     CalibArgs a;

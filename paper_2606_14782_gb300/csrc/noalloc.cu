@@ -4,16 +4,15 @@
 // HBM for its KV cache up front and forbids side allocations, or code that
 // must not pay the implicit device-wide synchronisation of cudaMalloc /
 // cudaFree in the middle of prefill.  For them, bacon_window_scores_noalloc
-// runs the same three window kernels as the context-based calls, but keeps
-// their scratch (pass-1 partial statistics and the per-row normalisers) in
-// one file-scope __device__ array instead of
-// context-owned buffers.
+// runs the same window kernels as the context-based calls, but keeps
+// their scratch (pass-1 partial statistics) in one file-scope __device__
+// array instead of context-owned buffers.
 //
 // The call returns before its kernels run, so a device-side failure (a
 // bounded pipeline wait that ran out) cannot come back as its status.  The
-// same array holds an error word for that: each call clears it, the window
-// kernels latch a timeout in it, and a last small kernel fills B, Q and E
-// with NaN when it is set, so that a caller never reads partial scores as
+// same array holds an error word for that: the window kernels latch a timeout
+// in it, and a last small kernel, when it is set, fills B, Q and E with NaN
+// and clears it, so that a caller never reads partial scores as
 // valid ones.
 #include <atomic>
 #include <cstdlib>
@@ -36,11 +35,10 @@ constexpr int kMaxDevices = 64;
 
 constexpr int kErrSlots = 2;          // 16 bytes holding the error word
 
-// [units][chunks][rows] partial (max, sum) pairs, then [units][rows] fp32
-// normalisers packed two per float2, then the device error word.  About
-// 528 KiB, held by every GPU that loads the library until the process exits.
-static __device__ __align__(256) float2
-    g_scratch[kMaxTotalRows * kMaxChunks + kMaxTotalRows / 2 + kErrSlots];
+// [units][chunks][rows] partial (max, sum) pairs, then the device error word.
+// About 512 KiB, held by every GPU that loads the library until the process
+// exits.
+static __device__ __align__(256) float2 g_scratch[kMaxTotalRows * kMaxChunks + kErrSlots];
 
 std::mutex g_setup_mutex;
 void* g_scratch_addr[kMaxDevices] = {};
@@ -61,17 +59,21 @@ int take_fault()
     return g_fault_pending.compare_exchange_strong(one, 0) ? 1 : 0;
 }
 
-// B, Q and E become NaN when a window kernel of this call latched an error.
-__global__ void poison_on_error_kernel(const int* err, float* B, float* Q, float* E, size_t n)
+// B, Q and E become NaN when a window kernel of this call latched an error,
+// and the error word is cleared for the next call (one block: it has nothing
+// to do unless a wait ran out, and the clearing needs no launch of its own).
+__global__ void __launch_bounds__(1024)
+poison_on_error_kernel(int* err, float* B, float* Q, float* E, size_t n)
 {
     if (*reinterpret_cast<const volatile int*>(err) == 0) return;
     const float nan = __int_as_float(0x7fc00000);
-    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-         i += (size_t)gridDim.x * blockDim.x) {
+    for (size_t i = threadIdx.x; i < n; i += blockDim.x) {
         B[i] = nan;
         Q[i] = nan;
         E[i] = nan;
     }
+    __syncthreads();
+    if (threadIdx.x == 0) *err = 0;
 }
 
 }  // namespace
@@ -122,9 +124,7 @@ bacon_status bacon_window_scores_noalloc(int kv_heads, int q_heads, int head_dim
     s.rows = (int)rows;
     const int chunks = (seq_len + kChunk - 1) / kChunk;
     float2* partial = scratch;
-    float* lse2 = reinterpret_cast<float*>(scratch + (size_t)kMaxTotalRows * kMaxChunks);
-    int* err = reinterpret_cast<int*>(scratch + (size_t)kMaxTotalRows * kMaxChunks +
-                                      kMaxTotalRows / 2);
+    int* err = reinterpret_cast<int*>(scratch + (size_t)kMaxTotalRows * kMaxChunks);
     const long long krows = (long long)kv_heads * seq_len, qrows = (long long)q_heads * window;
     TcArgs a;
     TcMaps m;  // the TMA descriptors are kernel parameters
@@ -132,14 +132,12 @@ bacon_status bacon_window_scores_noalloc(int kv_heads, int q_heads, int head_dim
         !encode_rows_map(&m.q, q_win, head_dim, qrows, 1, qrows * head_dim * 2, kTcQBoxRows))
         return BACON_ECUDA;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    // the error word must start at zero for this call
-    if (cudaMemsetAsync(err, 0, sizeof(int), st) != cudaSuccess) return BACON_ECUDA;
     a.kmaps = a.qmaps = nullptr;
     a.s = s;
     a.chunks = chunks;
     a.total_chunks = s.units * chunks;
     a.partial = partial;
-    a.lse2 = lse2;
+    a.lse2 = nullptr;  // pass 2 forms the row normalisers from the partials
     a.B = B_out;
     a.Q = Q_out;
     a.E = E_out;
@@ -147,15 +145,14 @@ bacon_status bacon_window_scores_noalloc(int kv_heads, int q_heads, int head_dim
     TcArgs a1 = a;
     a1.fault = take_fault();
     cudaError_t e = launch_window_stats_tc(a1, m, st);
-    if (e == cudaSuccess) e = launch_window_combine(s, chunks, partial, lse2, st);
     if (e == cudaSuccess) e = launch_window_scores_tc(a, m, st);
     if (e == cudaSuccess) {
-        const size_t n = (size_t)kv_heads * seq_len;
-        const size_t blocks = (n + 255) / 256;
-        poison_on_error_kernel<<<(unsigned)(blocks < 1024 ? blocks : 1024), 256, 0, st>>>(
-            err, B_out, Q_out, E_out, n);
+        poison_on_error_kernel<<<1, 1024, 0, st>>>(err, B_out, Q_out, E_out,
+                                                   (size_t)kv_heads * seq_len);
         e = cudaGetLastError();
     }
+    // without that kernel, what this call latched must not reach the next one
+    if (e != cudaSuccess) cudaMemsetAsync(err, 0, sizeof(int), st);
     return e == cudaSuccess ? BACON_OK : BACON_ECUDA;
 }
 

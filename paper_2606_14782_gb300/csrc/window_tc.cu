@@ -229,37 +229,86 @@ __device__ __forceinline__ uint32_t sw128_offset(int row, int col)
                       ((col * 2) & 15));
 }
 
-// Pass 2 bias operand of unit u: for job j and its row l (window row
-// row0_j + l), columns 16 j .. 16 j + 2 hold -lse2 / c as three bf16 parts
-// whose sum is the fp32 value to about 2^-24; rows beyond the window rows
-// get a huge negative bias so their exponentials vanish.  Written by the 32
-// lanes of the producer warp; columns 16 j + 3 .. stay zero.
-__device__ __forceinline__ void write_bias(const TcArgs& a, uint8_t* bias, int u, const JobTable& jt,
-                                           float inv_c)
+// log2 of one window row's softmax normaliser over all chunks, plus
+// log2(G W), so that pass 2's 2^(logit' - lse2) is A_{q,i} / (G W).  p: the
+// row's partials, `rows` apart.
+__device__ __forceinline__ float combine_row(const float2* __restrict__ p, int chunks, int rows)
+{
+    float M = -INFINITY;
+#pragma unroll 8
+    for (int c = 0; c < chunks; ++c) M = fmaxf(M, p[(size_t)c * rows].x);
+    float Z = 0.f;
+#pragma unroll 8
+    for (int c = 0; c < chunks; ++c) {
+        const float2 v = p[(size_t)c * rows];
+        if (v.y > 0.f) Z += v.y * exp2f(v.x - M);
+    }
+    return M + log2f(Z) + log2f((float)rows);
+}
+
+// Pass 2's accumulator bias of window row r of unit u: -lse2 / c, or a huge
+// negative value (whose exponentials vanish) beyond the window rows.
+__device__ __forceinline__ float row_bias(const TcArgs& a, int u, int r, float inv_c)
 {
     const Shape& s = a.s;
-    const int lane = threadIdx.x & 31;
+    if (r >= s.rows) return -1.0e38f;
+    const float lse2 = a.lse2 ? a.lse2[(size_t)u * s.rows + r]
+                              : combine_row(a.partial + (size_t)u * a.chunks * s.rows + r,
+                                            a.chunks, s.rows);
+    return -lse2 * inv_c;
+}
+
+// Pass 2 bias operand: for job j and its row l (window row row0_j + l),
+// columns 16 j .. 16 j + 2 hold the row's bias as three bf16 parts whose sum
+// is the fp32 value to about 2^-24; columns 16 j + 3 .. stay zero.
+__device__ __forceinline__ void write_bias_row(uint8_t* bias, const JobTable& jt, int r, float x)
+{
+    int j = 0;
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        if (j >= jt.n_jobs) break;
-        for (int l = lane; l < jt.n(j); l += 32) {
-            const int r = jt.row0(j) + l;
-            const float x = r < s.rows ? -a.lse2[(size_t)u * s.rows + r] * inv_c : -1.0e38f;
-            const __nv_bfloat16 hi = __float2bfloat16_rn(x);
-            const float r1 = x - __bfloat162float(hi);
-            const __nv_bfloat16 mid = __float2bfloat16_rn(r1);
-            const __nv_bfloat16 lo = __float2bfloat16_rn(r1 - __bfloat162float(mid));
-            const uint32_t off = sw128_offset(l, 16 * j);
-            *reinterpret_cast<uint32_t*>(bias + off) =
-                (uint32_t)__bfloat16_as_ushort(hi) | ((uint32_t)__bfloat16_as_ushort(mid) << 16);
-            *reinterpret_cast<uint32_t*>(bias + off + 4) = (uint32_t)__bfloat16_as_ushort(lo);
+    for (int i = 1; i < 4; ++i)
+        if (i < jt.n_jobs && r >= jt.row0(i)) j = i;
+    const __nv_bfloat16 hi = __float2bfloat16_rn(x);
+    const float r1 = x - __bfloat162float(hi);
+    const __nv_bfloat16 mid = __float2bfloat16_rn(r1);
+    const __nv_bfloat16 lo = __float2bfloat16_rn(r1 - __bfloat162float(mid));
+    const uint32_t off = sw128_offset(r - jt.row0(j), 16 * j);
+    *reinterpret_cast<uint32_t*>(bias + off) =
+        (uint32_t)__bfloat16_as_ushort(hi) | ((uint32_t)__bfloat16_as_ushort(mid) << 16);
+    *reinterpret_cast<uint32_t*>(bias + off + 4) = (uint32_t)__bfloat16_as_ushort(lo);
+}
+
+// The bias operand of unit u, by the 32 lanes of the producer warp (the
+// normalisers of a lane's rows are loaded eight at a time).
+__device__ __forceinline__ void write_bias(const TcArgs& a, uint8_t* bias, int u, const JobTable& jt,
+                                           int granules, float inv_c)
+{
+    const int lane = threadIdx.x & 31, total = 16 * granules;
+    if (!a.lse2) {
+#pragma unroll 1
+        for (int r = lane; r < total; r += 32) write_bias_row(bias, jt, r, row_bias(a, u, r, inv_c));
+        return;
+    }
+    const float* lse2 = a.lse2 + (size_t)u * a.s.rows;
+#pragma unroll 1
+    for (int r0 = lane; r0 < total; r0 += 256) {
+        float x[8];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+            const int r = r0 + 32 * e;
+            x[e] = r < a.s.rows ? -lse2[r] * inv_c : -1.0e38f;
+        }
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+            const int r = r0 + 32 * e;
+            if (r < total) write_bias_row(bias, jt, r, x[e]);
         }
     }
 }
 
 // All 32 lanes run the loop; lane 0 issues the copies.  At each new unit the
 // window rows are reloaded once the previous unit's MMAs have released them
-// (pass 2 also rewrites the bias operand, a second arrival on q_full).
+// (pass 2 also rewrites the bias operand, a second arrival on q_full; the
+// CTA's first unit has its bias from the kernel's prologue).
 template <int D, int PASS>
 __device__ __forceinline__ void produce(const TcArgs& a, const TcMaps& maps, const Plan& pl,
                                         const Smem& L, uint8_t* sm, const Bars& b,
@@ -299,9 +348,11 @@ __device__ __forceinline__ void produce(const TcArgs& a, const TcMaps& maps, con
                                         h * s.rows + r0 + i * kQBox, qz, b.q_full(slot));
             }
             if (PASS == 2) {
-                write_bias(a, sm + L.bias + slot * L.bias_slot, u, jt, inv_c);
-                tc::fence_proxy_async_smem();
-                __syncwarp();
+                if (qloads > 0) {
+                    write_bias(a, sm + L.bias + slot * L.bias_slot, u, jt, pl.granules, inv_c);
+                    tc::fence_proxy_async_smem();
+                    __syncwarp();
+                }
                 if (lane == 0) tc::mbar_arrive(b.q_full(slot));
             }
             ++qloads;
@@ -1004,24 +1055,15 @@ __device__ __forceinline__ void epilogue_scores(const TcArgs& a, const Plan& pl,
 
 // ------------------------------------------------------------------ merge
 
-// Per (unit, window row): log2 of the softmax normaliser over all chunks,
-// plus log2(G W), so that pass 2's 2^(logit' - lse2) is A_{q,i} / (G W).
+// Every unit's row normalisers (calls of many units: pass 2 would form a
+// unit's normalisers once per CTA that works on it).
 __global__ void window_combine_kernel(Shape s, int chunks, const float2* __restrict__ partial,
                                       float* __restrict__ lse2)
 {
     const int u = blockIdx.x;
-    const float log2_gw = log2f((float)s.rows);
-    for (int r = threadIdx.x; r < s.rows; r += blockDim.x) {
-        const float2* p = partial + (size_t)u * chunks * s.rows + r;
-        float M = -INFINITY;
-        for (int c = 0; c < chunks; ++c) M = fmaxf(M, p[(size_t)c * s.rows].x);
-        float Z = 0.f;
-        for (int c = 0; c < chunks; ++c) {
-            const float2 v = p[(size_t)c * s.rows];
-            if (v.y > 0.f) Z += v.y * exp2f(v.x - M);
-        }
-        lse2[(size_t)u * s.rows + r] = M + log2f(Z) + log2_gw;
-    }
+    for (int r = threadIdx.x; r < s.rows; r += blockDim.x)
+        lse2[(size_t)u * s.rows + r] =
+            combine_row(partial + (size_t)u * chunks * s.rows + r, chunks, s.rows);
 }
 
 // Row normalisers supplied by the caller's prefill attention: per (request,
@@ -1071,6 +1113,19 @@ __global__ void __launch_bounds__(kThreads, 1) window_tc_kernel(TcArgs a, Plan p
         tc::st_shared_volatile(b.abort(), 0u);
         tc::fence_barrier_init();
     }
+    // The producer starts its loads once the barriers exist; the other warps
+    // meet it at barrier 1, which it only arrives at: the first tiles and
+    // window rows come in while tensor memory is allocated and the first
+    // unit's bias is formed (by all 512 epilogue threads, a row each, where
+    // one warp took 14 dependent rounds).  With the row normalisers formed
+    // here instead of by a launch of their own, the passes of one layer (4
+    // kv-heads x 448 rows x 16384 tokens) take 38 instead of 51 us; later
+    // units' normalisers loaded together: pass 2 of 448 units 579 -> 563 us.
+    if (warp == 0) {
+        __syncwarp();
+        tc::named_barrier_arrive(1, kThreads);
+        produce<D, PASS>(a, maps, pl, L, sm, b, jt);
+    }
     if (threadIdx.x == 32) {
         if (!a.kmaps) tc::tma_prefetch_desc(&maps.k);
         if (!a.qmaps) tc::tma_prefetch_desc(&maps.q);
@@ -1080,38 +1135,42 @@ __global__ void __launch_bounds__(kThreads, 1) window_tc_kernel(TcArgs a, Plan p
         tc::tmem_alloc(b.tmem_slot(), kTmemCols);
         tc::tmem_relinquish();
     }
-    if (PASS == 2 && threadIdx.x >= 64 && threadIdx.x < 64 + 128) {
+    if (PASS == 2 && warp >= 2) {
         // constant operand: 1 in columns 0-2 of every token row (one atom of
-        // 8 rows when ones_atom); the bias operand starts zeroed (the
-        // producer fills columns 16 j .. 16 j + 2)
+        // 8 rows when ones_atom); the bias operand starts zeroed, then takes
+        // the first unit's values (the producer rewrites it for later units)
         const int row = threadIdx.x - 64;
-        for (int rr = row; rr < pl.q_slots * pl.bias_rows; rr += 128) {
-            uint4* bias = reinterpret_cast<uint4*>(sm + L.bias + rr * 128);
-            for (int q = 0; q < 8; ++q) bias[q] = make_uint4(0u, 0u, 0u, 0u);
-        }
-        if (!pl.ones_atom || row < 8) {
+        int g0, g1;
+        item_range(a.items, &g0, &g1);
+        const int u = g0 / ((a.s.N + kTileTok - 1) / kTileTok);
+        const float x = row < 16 * pl.granules ? row_bias(a, u, row, sqrtf((float)D) / kLog2e) : 0.f;
+        for (int i = row; i < pl.q_slots * pl.bias_rows * 8; i += kEpiThreads)
+            reinterpret_cast<uint4*>(sm + L.bias)[i] = make_uint4(0u, 0u, 0u, 0u);
+        if (row < (pl.ones_atom ? 8 : 128)) {
             uint4* ones = reinterpret_cast<uint4*>(sm + L.ones + row * 128);
             for (int q = 0; q < 8; ++q) ones[q] = make_uint4(0u, 0u, 0u, 0u);
             uint8_t* r = sm + L.ones + sw128_offset(row, 0);
             *reinterpret_cast<uint32_t*>(r) = 0x3F803F80u;  // bf16 1.0, 1.0
             *reinterpret_cast<uint32_t*>(r + 4) = 0x00003F80u;
         }
+        tc::named_barrier_sync(2, kEpiThreads);  // the zeros come first
+        if (row < 16 * pl.granules) write_bias_row(sm + L.bias, jt, row, x);
         tc::fence_proxy_async_smem();
     }
-    tc::fence_before_sync();
-    __syncthreads();
-    tc::fence_after_sync();
+    if (warp != 0) {
+        tc::fence_before_sync();
+        tc::named_barrier_sync(1, kThreads);
+        tc::fence_after_sync();
+    }
 
-    if (warp == 0) {
-        produce<D, PASS>(a, maps, pl, L, sm, b, jt);
-    } else if (warp == 1) {
+    if (warp == 1) {
         if (tc::elect_one()) {
             if (pl.nbuf_log2 == 1)
                 issue<D, PASS, 1>(a, pl, L, sm, b, jt);
             else
                 issue<D, PASS, 2>(a, pl, L, sm, b, jt);
         }
-    } else {
+    } else if (warp >= 2) {
         if (PASS == 1)
         {
             const int nrb = pl.blocks;

@@ -33,7 +33,7 @@ struct TcArgs {
     int total_chunks;          // units * chunks
     int items;                 // work items of the launch (set by it)
     float2* partial;           // pass 1 output [units][chunks][rows]
-    const float* lse2;         // pass 2 input  [units][rows]
+    const float* lse2;         // pass 2 input  [units][rows]; null: from `partial`
     float* B;                  // pass 2 outputs [units][N]
     float* Q;
     float* E;
