@@ -10,17 +10,23 @@
 // the k-th best key and how many of the keys equal to it are taken; the
 // members are then decided thread by thread in position order.
 //
-// Each thread owns PER consecutive positions [t PER, t PER + PER), so the
-// pooling and coherence windows slide along a thread's own positions and
-// the position order of the members is (thread, slot) order: one
-// block-wide exclusive scan gives every thread its tie rank or its output
-// offset.  The one per-position array in shared memory (the pooled
-// backbone, then the final score: the keys of the two selections) is
-// stored slot-major, element (slot k, thread t) at k T + t, so the radix
-// select's passes, which walk the storage index s = k T + t, read
-// consecutive words, and those are the thread's own slots.  V lives in
-// registers; the windows' neighbours come from the adjacent lanes' runs by
-// warp shuffles (from global memory at a warp's two ends).
+// Each thread owns PER consecutive positions, [t PER, t PER + PER), and
+// keeps them in registers: the pooled backbone and then the final score (the
+// keys of the two selections), and V.  The windows' neighbours come from the
+// adjacent lanes' runs by warp shuffles (from global memory at a warp's two
+// ends), and position order is (thread, slot) order, so one block-wide
+// exclusive scan gives every thread its tie rank or its output offset.
+//
+// A unit is bound by latency: about 15 dependent rounds of a block barrier
+// each, one CTA per unit and at most one or two CTAs' worth of warps per SM.
+// Keys in registers take the passes over all of them off shared memory, the
+// boundary bin's keys are ranked by counting instead of a second histogram
+// and a warp's sort, every warp finishes the block reductions itself (one
+// barrier each instead of three), and runs of 8 positions load B and every
+// residual they need at once.  With a shared-memory array of keys, two
+// histogram passes and about 30 barriers: 110 -> 77 us (448 units x 16384
+// tokens), 25 -> 17.5 (112 x 6528), 21 -> 14 (112 x 4096), 24 -> 14 (1024 x
+// 1024).
 //
 // The standard deviations are fp32 sums over the members: B~'s moments
 // about the M-th value (one walk), V's mean and then its squared
@@ -42,43 +48,39 @@ using namespace sel;
 // 16384 tokens and of 24 up to 24576.
 constexpr int kMaxPrompt = 24576;
 
-// Four block-wide fp32 sums in one round (red holds 4 x 33 floats), by a
-// shuffle tree (pairwise, so the rounding error grows with log2 of the
-// count).  FP64 is avoided: its rate on this part is a small fraction of fp32.
-__device__ float4 block_sum4(float4 v, float* red)
+// Block-wide fp32 sums of NV values in one round, by a shuffle tree (pairwise,
+// so the rounding error grows with log2 of the count).  Every warp reduces
+// the warps' sums itself, so a round costs one block barrier; `red` holds
+// NV x 32 floats and is not used again before the next barrier.  FP64 is
+// avoided: its rate on this part is a small fraction of fp32.
+template <int T, int NV>
+__device__ __forceinline__ void block_sums(float (&v)[NV], float* red)
 {
+    constexpr int kWarps = T / 32;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        v.x += __shfl_xor_sync(0xffffffffu, v.x, o);
-        v.y += __shfl_xor_sync(0xffffffffu, v.y, o);
-        v.z += __shfl_xor_sync(0xffffffffu, v.z, o);
-        v.w += __shfl_xor_sync(0xffffffffu, v.w, o);
-    }
-    if (lane == 0) {
-        red[warp] = v.x;
-        red[33 + warp] = v.y;
-        red[66 + warp] = v.z;
-        red[99 + warp] = v.w;
-    }
-    __syncthreads();
-    if (warp < 4) {
-        const int nw = (int)(blockDim.x >> 5);
-        float t = lane < nw ? red[33 * warp + lane] : 0.f;
+    for (int o = 16; o > 0; o >>= 1)
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-        if (lane == 0) red[33 * warp + 32] = t;
-    }
+        for (int i = 0; i < NV; ++i) v[i] += __shfl_xor_sync(0xffffffffu, v[i], o);
+    if (lane == 0)
+#pragma unroll
+        for (int i = 0; i < NV; ++i) red[32 * i + warp] = v[i];
     __syncthreads();
-    const float4 tot = make_float4(red[32], red[65], red[98], red[131]);
-    __syncthreads();
-    return tot;
+#pragma unroll
+    for (int i = 0; i < NV; ++i) v[i] = lane < kWarps ? red[32 * i + lane] : 0.f;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+        for (int i = 0; i < NV; ++i) v[i] += __shfl_xor_sync(0xffffffffu, v[i], o);
 }
 
-// Exclusive prefix sum of one int per thread, in thread order; *total
-// receives the sum.  warp_sums holds 32 ints.
-__device__ int block_exclusive_scan(int v, int* warp_sums, int* total)
+// Exclusive prefix sum of one int per thread, in thread order; total receives
+// the sum.  One block barrier: every warp scans the warps' sums itself.
+// warp_sums holds 32 ints and is not used again before the next barrier.
+template <int T>
+__device__ __forceinline__ int block_exclusive_scan(int v, int* warp_sums, int& total)
 {
+    constexpr int kWarps = T / 32;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     int incl = v;
 #pragma unroll
@@ -88,22 +90,15 @@ __device__ int block_exclusive_scan(int v, int* warp_sums, int* total)
     }
     if (lane == 31) warp_sums[warp] = incl;
     __syncthreads();
-    if (warp == 0) {
-        const int nw = (int)(blockDim.x >> 5);
-        const int w = lane < nw ? warp_sums[lane] : 0;
-        int wi = w;
+    const int w = lane < kWarps ? warp_sums[lane] : 0;
+    int wi = w;
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int y = __shfl_up_sync(0xffffffffu, wi, o);
-            if (lane >= o) wi += y;
-        }
-        if (lane < nw) warp_sums[lane] = wi - w;
-        if (lane == 31) *total = wi;
+    for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, wi, o);
+        if (lane >= o) wi += y;
     }
-    __syncthreads();
-    const int r = warp_sums[warp] + incl - v;
-    __syncthreads();
-    return r;
+    total = __shfl_sync(0xffffffffu, wi, 31);
+    return __shfl_sync(0xffffffffu, wi - w, warp) + incl - v;
 }
 
 // Ask L2 to fetch the n floats at p (one prefetch per 128-byte line, every
@@ -151,44 +146,20 @@ __device__ __forceinline__ void store_run(float* dst, int i0, int n, const float
     }
 }
 
-// Slot-major shared-memory array of T threads x PER positions.
-template <int T, int PER>
-struct Slots {
-    float* a;
-    // storage index of position i, and the position held at storage index s
-    __device__ static __forceinline__ int at(int i) { return (i % PER) * T + i / PER; }
-    __device__ static __forceinline__ int pos(int s) { return (s % T) * PER + s / T; }
-    __device__ __forceinline__ float& own(int k) const { return a[k * T + (int)threadIdx.x]; }
-    __device__ __forceinline__ float operator[](int i) const { return a[at(i)]; }
-};
-
-// Keys of the candidates [0, n_cand) of a slot-major array, walked by
-// storage index (the radix select's passes read consecutive words).
-template <int T, int PER>
-struct SlotKeys {
-    const float* a;
-    int n_cand;
-    __device__ __forceinline__ bool operator()(int s, uint32_t& key) const
-    {
-        if (Slots<T, PER>::pos(s) >= n_cand) return false;
-        key = float_key(a[s]);
-        return true;
-    }
-};
-
-// Membership of the thread's candidates in the k best (bit k of the result):
-// key > tau, or key == tau among the first `need` such keys in position
-// order.  eq_before = keys equal to tau at lower positions (other threads).
-template <int T, int PER>
-__device__ __forceinline__ uint32_t members(const Slots<T, PER>& arr, int i0, int n_cand,
-                                            const SelectResult& sel, int eq_before)
+// Membership of the thread's candidates (its first nv slots) in the k best
+// (bit k of the result): key > tau, or key == tau among the first `need` such
+// keys in position order.  eq_before = keys equal to tau at lower positions
+// (other threads).
+template <int PER>
+__device__ __forceinline__ uint32_t members(const float* x, int nv, const SelectResult& sel,
+                                            int eq_before)
 {
     uint32_t m = 0u;
     int rank = eq_before;
 #pragma unroll
     for (int k = 0; k < PER; ++k) {
-        if (i0 + k < n_cand) {
-            const uint32_t key = float_key(arr.own(k));
+        if (k < nv) {
+            const uint32_t key = float_key(x[k]);
             const bool eq = key == sel.tau;
             if (key > sel.tau || (eq && rank < sel.need)) m |= 1u << k;
             rank += eq;
@@ -200,15 +171,14 @@ __device__ __forceinline__ uint32_t members(const Slots<T, PER>& arr, int i0, in
 // Keys equal to tau at lower positions than this thread's run (0 without a
 // scan when every tie is taken: membership then never needs the rank).
 template <int T, int PER>
-__device__ __forceinline__ int ties_before(const Slots<T, PER>& arr, int i0, int n_cand,
-                                           const SelectResult& sel, int* warp_sums, int* total)
+__device__ __forceinline__ int ties_before(const float* x, int nv, const SelectResult& sel,
+                                           int* warp_sums)
 {
     if (sel.all_ties_in()) return 0;
-    int eq = 0;
+    int eq = 0, total;
 #pragma unroll
-    for (int k = 0; k < PER; ++k)
-        eq += (i0 + k < n_cand) && float_key(arr.own(k)) == sel.tau;
-    return block_exclusive_scan(eq, warp_sums, total);
+    for (int k = 0; k < PER; ++k) eq += k < nv && float_key(x[k]) == sel.tau;
+    return block_exclusive_scan<T>(eq, warp_sums, total);
 }
 
 // The residual E of the thread's run into x (0 at and past N), added to v
@@ -320,27 +290,122 @@ __device__ __forceinline__ void residual_and_coherence(const float* __restrict__
     coherence_any<PER>(Ec, i0, N, r, v);
 }
 
+// The evidence V = E + L + T of the thread's run (Eqs. 5-11) into v, 0 at and
+// past N; x is scratch for PER floats.  E_of(j) is layer j's residuals.
+template <int PER, typename EFn>
+__device__ __forceinline__ void evidence_run(const Calib& c, EFn E_of, int layer, int i0, int N,
+                                             float* x, float* v)
+{
+    const float* Ec = E_of(layer);
+#pragma unroll
+    for (int k = 0; k < PER; ++k) v[k] = 0.f;
+    // persistence: mean of E over the preceding min(m, l) layers (Eqs. 8-9)
+    if (c.use_T) {
+        const int nprev = min(c.m, layer);
+        const float inv_prev = nprev > 0 ? 1.f / (float)nprev : 0.f;
+        // a layer's run in chunks of at most 16 (V and one chunk in registers)
+        constexpr int CH = PER <= 16 ? PER : PER / 2;
+        static_assert(PER % CH == 0 && CH % 4 == 0, "chunks of whole 16-byte loads");
+        constexpr int kAhead = PER <= 8 ? 4 : 1;  // layers whose loads are in flight together
+#pragma unroll kAhead
+        for (int j = layer - nprev; j < layer; ++j) {
+#pragma unroll
+            for (int c0 = 0; c0 < PER; c0 += CH) {
+                float e[CH];
+                load_run<CH>(E_of(j), i0 + c0, N, e);
+#pragma unroll
+                for (int k = 0; k < CH; ++k) v[c0 + k] += e[k];
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < PER; ++k) v[k] *= inv_prev;
+    }
+    // E, and the coherence: truncated radius-r box mean of E (Eqs. 5-7)
+    if (c.use_L) {
+        residual_and_coherence<PER>(Ec, i0, N, c.r, c.use_E, x, v);
+    } else if (c.use_E) {
+        load_run<PER>(Ec, i0, N, x);
+#pragma unroll
+        for (int k = 0; k < PER; ++k) v[k] += x[k];
+    }
+#pragma unroll
+    for (int k = 0; k < PER; ++k)
+        if (i0 + k >= N) v[k] = 0.f;
+}
+
+// The pooled backbone of the thread's run (max over [i - half, i + half] of
+// the candidates, 0 past them) from Bu's run in b, in place; the key range of
+// the candidates goes to kmin, kmax.
+template <int PER>
+__device__ __forceinline__ void pool_run(const float* __restrict__ Bu, int i0, int n_cand, int half,
+                                         float* b, uint32_t& kmin, uint32_t& kmax)
+{
+    float p[PER];
+    if (half == 3) {
+        // width 7 (the default): the run and three positions either side in
+        // registers (-inf outside the candidates; the neighbours' values by
+        // shuffles, from global memory at a warp's two ends), each output a
+        // maximum of seven by three max3
+        const int lane = threadIdx.x & 31;
+        float hl[3], hr[3];
+#pragma unroll
+        for (int m = 0; m < 3; ++m) {
+            const int jl = i0 - 3 + m, jr = i0 + PER + m;
+            hl[m] = (lane == 0 && jl >= 0 && jl < n_cand) ? __ldg(Bu + jl) : -INFINITY;
+            hr[m] = (lane == 31 && jr < n_cand) ? __ldg(Bu + jr) : -INFINITY;
+        }
+#pragma unroll
+        for (int k = 0; k < PER; ++k)
+            if (i0 + k >= n_cand) b[k] = -INFINITY;
+#pragma unroll
+        for (int m = 0; m < 3; ++m) {
+            const float lo = __shfl_up_sync(0xffffffffu, b[PER - 3 + m], 1);
+            const float hi = __shfl_down_sync(0xffffffffu, b[m], 1);
+            if (lane != 0) hl[m] = lo;
+            if (lane != 31) hr[m] = hi;
+        }
+        auto at = [&](int j) -> float { return j < 0 ? hl[j + 3] : (j >= PER ? hr[j - PER] : b[j]); };
+#pragma unroll
+        for (int k = 0; k < PER; ++k)
+            p[k] = max3f(max3f(at(k - 3), at(k - 2), at(k - 1)), max3f(at(k), at(k + 1), at(k + 2)),
+                         at(k + 3));
+    } else {
+#pragma unroll
+        for (int k = 0; k < PER; ++k) {
+            const int i = i0 + k;
+            p[k] = -INFINITY;
+            if (i < n_cand) {
+                const int lo = max(0, i - half), hi = min(n_cand - 1, i + half);
+                for (int v = lo; v <= hi; ++v) p[k] = fmaxf(p[k], __ldg(Bu + v));
+            }
+        }
+    }
+#pragma unroll
+    for (int k = 0; k < PER; ++k) {
+        b[k] = 0.f;
+        if (i0 + k < n_cand) {
+            b[k] = p[k];
+            kmin = min(kmin, float_key(p[k]));
+            kmax = max(kmax, float_key(p[k]));
+        }
+    }
+}
+
 // One unit (request, layer, kv-head) u under hyper-parameters c.  lam_out
 // (may be null) receives lambda; idx_pair is the pair's [Hkv][kept] output.
-// N <= T PER.  One slot-major array in shared memory holds the pooled
-// backbone and then the final score; V stays in the thread's registers
-// (every later read of it is the thread's own), and the pooling and
-// coherence windows read their neighbours from global memory (L1), so a
-// unit needs T PER floats of shared memory and two CTAs share an SM at the
-// 512-thread classes.
+// N <= T PER.  The thread's run of the pooled backbone (then of the final
+// score: the keys of the two selections) stays in registers, and so does V
+// where a run is 8 positions; longer runs form V after the first selection,
+// with the backbone parked in the thread's own column of shared memory.
 template <int T, int PER>
 __device__ __forceinline__ void calibrate_unit(const Shape& s, const Calib& c, const CalibArgs& a,
                                                int u, float* lam_out, int32_t* idx_pair)
 {
-    extern __shared__ __align__(16) float sm[];
-    const Slots<T, PER> A{sm};  // pooled backbone B~, then the final score S
-    // the selections never look at more than T PER keys
-    constexpr int kCap = T * PER < kSelCap ? T * PER : kSelCap;
-    __shared__ __align__(16) int hist[sel_hist_ints(kCap)];
-    __shared__ int bcast[8];
-    __shared__ int warp_sums[32];
-    __shared__ float red[4 * 33];
-    __shared__ int total_s;
+    constexpr bool kPark = PER > 8;
+    extern __shared__ __align__(16) float sm[];  // kPark: [PER][T]
+    __shared__ SelectScratch<T> sel_sm;
+    __shared__ int ties[2][32], offsets[32];
+    __shared__ float red_b[3 * 32], red_v[32];
 
     const int N = s.N, W = s.W;
     const int pair = u / s.hkv, h = u - pair * s.hkv;
@@ -351,132 +416,50 @@ __device__ __forceinline__ void calibrate_unit(const Shape& s, const Calib& c, c
     const int kept_total = min(a.budget[pair], N);
     const int keep = kept_total - win;
     const int i0 = (int)threadIdx.x * PER;
+    const int nv = max(0, min(PER, n_cand - i0));  // this thread's candidates
 
+    float b[PER];  // pooled backbone B~, then the final score S
     uint32_t skmin = 0xffffffffu, skmax = 0u;  // key range of S over the candidates
-    auto Eof = [&](int j) -> const float* {
+    auto E_of = [&](int j) -> const float* {
         return a.Ering + (long long)rq * a.ring_req_stride +
                (long long)(j % a.ring) * s.hkv * N + (long long)h * N;
     };
 
     if (a.compute_scores) {
         const float* Bu = a.B + (size_t)u * N;
-        const float* Ec = Eof(layer);
-        const int nprev = min(c.m, layer);
-        const float inv_prev = nprev > 0 ? 1.f / (float)nprev : 0.f;
-        // the residuals are read only after the pooling and the first
-        // selection: start bringing them into L2 now
-        prefetch_l2(Ec, N);
-        if (c.use_T)
-            for (int j = layer - nprev; j < layer; ++j) prefetch_l2(Eof(j), N);
-
-        // ---- pooled backbone over the candidates (max over [i - half, i + half])
-        float x[PER];
-        load_run<PER>(Bu, i0, N, x);
-        uint32_t kmin = 0xffffffffu, kmax = 0u;  // key range of B~ over the candidates
-        const int half = c.pool / 2;
-        if (half == 3) {
-            // width 7 (the default): the run and three positions either side
-            // in registers (-inf outside the candidates; the neighbours'
-            // values by shuffles, from global memory at a warp's two ends),
-            // each output a maximum of seven by three max3
-            const int lane = threadIdx.x & 31;
-            float hl[3], hr[3];
-#pragma unroll
-            for (int m = 0; m < 3; ++m) {
-                const int jl = i0 - 3 + m, jr = i0 + PER + m;
-                hl[m] = (lane == 0 && jl >= 0 && jl < n_cand) ? __ldg(Bu + jl) : -INFINITY;
-                hr[m] = (lane == 31 && jr < n_cand) ? __ldg(Bu + jr) : -INFINITY;
-            }
-#pragma unroll
-            for (int k = 0; k < PER; ++k)
-                if (i0 + k >= n_cand) x[k] = -INFINITY;
-#pragma unroll
-            for (int m = 0; m < 3; ++m) {
-                const float lo = __shfl_up_sync(0xffffffffu, x[PER - 3 + m], 1);
-                const float hi = __shfl_down_sync(0xffffffffu, x[m], 1);
-                if (lane != 0) hl[m] = lo;
-                if (lane != 31) hr[m] = hi;
-            }
-            auto at = [&](int j) -> float { return j < 0 ? hl[j + 3] : (j >= PER ? hr[j - PER] : x[j]); };
-#pragma unroll
-            for (int k = 0; k < PER; ++k) {
-                float mx = 0.f;
-                if (i0 + k < n_cand) {
-                    mx = max3f(max3f(at(k - 3), at(k - 2), at(k - 1)),
-                               max3f(at(k), at(k + 1), at(k + 2)), at(k + 3));
-                    kmin = min(kmin, float_key(mx));
-                    kmax = max(kmax, float_key(mx));
-                }
-                A.own(k) = mx;
-            }
+        float x[PER], v[PER];
+        load_run<PER>(Bu, i0, N, b);
+        if (kPark) {
+            // the residuals are read only after the first selection: start
+            // bringing them into L2 now
+            prefetch_l2(E_of(layer), N);
+            if (c.use_T)
+                for (int j = layer - min(c.m, layer); j < layer; ++j) prefetch_l2(E_of(j), N);
         } else {
-#pragma unroll
-            for (int k = 0; k < PER; ++k) {
-                const int i = i0 + k;
-                float mx = 0.f;
-                if (i < n_cand) {
-                    mx = -INFINITY;
-                    const int lo = max(0, i - half), hi = min(n_cand - 1, i + half);
-                    for (int v = lo; v <= hi; ++v) mx = fmaxf(mx, __ldg(Bu + v));
-                    kmin = min(kmin, float_key(mx));
-                    kmax = max(kmax, float_key(mx));
-                }
-                A.own(k) = mx;
-            }
+            evidence_run<PER>(c, E_of, layer, i0, N, x, v);
         }
-        if (a.Bp) {
-#pragma unroll
-            for (int k = 0; k < PER; ++k) x[k] = A.own(k);
-            store_run<PER>(a.Bp + (size_t)u * N, i0, N, x);
-        }
+        uint32_t kmin = 0xffffffffu, kmax = 0u;  // key range of B~ over the candidates
+        pool_run<PER>(Bu, i0, n_cand, c.pool / 2, b, kmin, kmax);
+        if (a.Bp) store_run<PER>(a.Bp + (size_t)u * N, i0, N, b);
 
-        // ---- the M best candidates by B~ (Eq. 12); V is computed after this
-        // selection, so that it is not held across it
+        // ---- the M best candidates by B~ (Eq. 12)
         const int calib_keep = min(a.calib_budget[pair], N) - win;
         const long long Ml = (long long)c.rho * (long long)(calib_keep > 0 ? calib_keep : 0);
         const int M = (int)(Ml < n_cand ? Ml : n_cand);
         uint32_t mem = 0u;
         float pb = 0.f;
         if (M > 0) {
-            const SelectResult sel = radix_select_range<kCap>(T * PER, M, SlotKeys<T, PER>{A.a, n_cand},
-                                                        hist, bcast, kmin, kmax);
-            const int eqb = ties_before(A, i0, n_cand, sel, warp_sums, &total_s);
-            mem = members(A, i0, n_cand, sel, eqb);
+            const SelectResult sel = select_runs<T, PER>(b, nv, M, sel_sm, kmin, kmax);
+            mem = members<PER>(b, nv, sel, ties_before<T, PER>(b, nv, sel, ties[0]));
             pb = key_float(sel.tau);
         }
-
-        // ---- persistence: mean of E over the preceding min(m, l) layers (Eqs. 8-9)
-        float v[PER];
+        if (kPark) {
 #pragma unroll
-        for (int k = 0; k < PER; ++k) v[k] = 0.f;
-        if (c.use_T) {
-            // a layer's run in chunks of at most 16 (V and one chunk in
-            // registers)
-            constexpr int CH = PER <= 16 ? PER : PER / 2;
-            static_assert(PER % CH == 0 && CH % 4 == 0, "chunks of whole 16-byte loads");
-            for (int j = layer - nprev; j < layer; ++j) {
+            for (int k = 0; k < PER; ++k) sm[k * T + threadIdx.x] = b[k];
+            evidence_run<PER>(c, E_of, layer, i0, N, x, v);
 #pragma unroll
-                for (int c0 = 0; c0 < PER; c0 += CH) {
-                    float e[CH];
-                    load_run<CH>(Eof(j), i0 + c0, N, e);
-#pragma unroll
-                    for (int k = 0; k < CH; ++k) v[c0 + k] += e[k];
-                }
-            }
-#pragma unroll
-            for (int k = 0; k < PER; ++k) v[k] *= inv_prev;
+            for (int k = 0; k < PER; ++k) b[k] = sm[k * T + threadIdx.x];
         }
-        // ---- E, and the coherence: truncated radius-r box mean of E (Eqs. 5-7)
-        if (c.use_L) {
-            residual_and_coherence<PER>(Ec, i0, N, c.r, c.use_E, x, v);
-        } else if (c.use_E) {
-            load_run<PER>(Ec, i0, N, x);
-#pragma unroll
-            for (int k = 0; k < PER; ++k) v[k] += x[k];
-        }
-#pragma unroll
-        for (int k = 0; k < PER; ++k)
-            if (i0 + k >= N) v[k] = 0.f;
         if (a.V) store_run<PER>(a.V + (size_t)u * N, i0, N, v);
 
         // ---- lambda over the M members (Eqs. 13-15).  B~ by moments about
@@ -485,29 +468,30 @@ __device__ __forceinline__ void calibrate_unit(const Shape& s, const Calib& c, c
         // square deviation from it (two reductions).
         float lam = 0.f;
         if (M > 0) {
-            float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+            float acc[3] = {0.f, 0.f, 0.f};
 #pragma unroll
             for (int k = 0; k < PER; ++k) {
                 if ((mem >> k) & 1u) {
-                    const float db = A.own(k) - pb;
-                    acc.x += db;
-                    acc.y = fmaf(db, db, acc.y);
-                    acc.z += v[k];
+                    const float db = b[k] - pb;
+                    acc[0] += db;
+                    acc[1] = fmaf(db, db, acc[1]);
+                    acc[2] += v[k];
                 }
             }
-            const float4 tot = block_sum4(acc, red);
+            block_sums<T, 3>(acc, red_b);
             const float inv_m = 1.f / (float)M;
-            const float mb = tot.x * inv_m, mv = tot.z * inv_m;
-            float4 dev = make_float4(0.f, 0.f, 0.f, 0.f);
+            const float mb = acc[0] * inv_m, mv = acc[2] * inv_m;
+            float dev[1] = {0.f};
 #pragma unroll
             for (int k = 0; k < PER; ++k) {
                 if ((mem >> k) & 1u) {
                     const float dv = v[k] - mv;
-                    dev.x = fmaf(dv, dv, dev.x);
+                    dev[0] = fmaf(dv, dv, dev[0]);
                 }
             }
-            const float varv = block_sum4(dev, red).x * inv_m;
-            const float stdb = sqrtf(fmaxf(tot.y * inv_m - mb * mb, 0.f));
+            block_sums<T, 1>(dev, red_v);
+            const float varv = dev[0] * inv_m;
+            const float stdb = sqrtf(fmaxf(acc[1] * inv_m - mb * mb, 0.f));
             const float stdv = sqrtf(varv);
             lam = c.gamma * stdb / (stdv + c.eps);
         }
@@ -515,48 +499,40 @@ __device__ __forceinline__ void calibrate_unit(const Shape& s, const Calib& c, c
         // ---- Eq. 16 over the candidates (0 elsewhere)
 #pragma unroll
         for (int k = 0; k < PER; ++k) {
-            float sv = 0.f;
-            if (i0 + k < n_cand) {
-                sv = fmaf(lam, v[k], A.own(k));
-                skmin = min(skmin, float_key(sv));
-                skmax = max(skmax, float_key(sv));
+            if (k < nv) {
+                b[k] = fmaf(lam, v[k], b[k]);
+                skmin = min(skmin, float_key(b[k]));
+                skmax = max(skmax, float_key(b[k]));
             }
-            A.own(k) = sv;
-            x[k] = sv;
         }
-        if (a.write_S) store_run<PER>(a.S + (size_t)u * N, i0, N, x);
-        __syncthreads();
+        if (a.write_S) store_run<PER>(a.S + (size_t)u * N, i0, N, b);
     } else {
-        float x[PER];
-        load_run<PER>(a.S + (size_t)u * N, i0, N, x);
+        load_run<PER>(a.S + (size_t)u * N, i0, N, b);
 #pragma unroll
         for (int k = 0; k < PER; ++k) {
-            A.own(k) = x[k];
-            if (i0 + k < n_cand) {
-                skmin = min(skmin, float_key(x[k]));
-                skmax = max(skmax, float_key(x[k]));
+            if (k < nv) {
+                skmin = min(skmin, float_key(b[k]));
+                skmax = max(skmax, float_key(b[k]));
             }
         }
-        __syncthreads();
     }
 
     if (!a.do_select) return;
     // ---- Eq. 17: the K best candidates by S, ascending, then the window
     int32_t* out = idx_pair + (size_t)h * kept_total;
     if (keep >= n_cand) {
-        for (int i = threadIdx.x; i < n_cand; i += blockDim.x) out[i] = i;
+        for (int i = threadIdx.x; i < n_cand; i += T) out[i] = i;
     } else if (keep > 0) {
-        const SelectResult sel = radix_select_range<kCap>(T * PER, keep, SlotKeys<T, PER>{A.a, n_cand},
-                                                    hist, bcast, skmin, skmax);
-        const int eqb = ties_before(A, i0, n_cand, sel, warp_sums, &total_s);
-        const uint32_t mem = members(A, i0, n_cand, sel, eqb);
-        int pos = block_exclusive_scan(__popc(mem), warp_sums, &total_s);
+        const SelectResult sel = select_runs<T, PER>(b, nv, keep, sel_sm, skmin, skmax);
+        const uint32_t mem = members<PER>(b, nv, sel, ties_before<T, PER>(b, nv, sel, ties[1]));
+        int total;
+        int pos = block_exclusive_scan<T>(__popc(mem), offsets, total);
 #pragma unroll
         for (int k = 0; k < PER; ++k)
             if ((mem >> k) & 1u) out[pos++] = i0 + k;
-        if (threadIdx.x == 0 && total_s != keep && a.err) atomicCAS(a.err, 0, 2);
+        if (threadIdx.x == 0 && total != keep && a.err) atomicCAS(a.err, 0, 2);
     }
-    for (int w = threadIdx.x; w < win; w += blockDim.x) out[keep + w] = N - W + w;
+    for (int w = threadIdx.x; w < win; w += T) out[keep + w] = N - W + w;
 }
 
 template <int T, int PER>
@@ -584,7 +560,7 @@ calibrate_sweep_kernel(Shape s, CalibTable t, CalibArgs a)
 template <int T, int PER>
 constexpr size_t smem_bytes()
 {
-    return (size_t)T * PER * sizeof(float);
+    return PER > 8 ? (size_t)T * PER * sizeof(float) : 0;
 }
 
 template <int T, int PER>

@@ -239,6 +239,153 @@ __device__ __noinline__ SelectResult radix_select_range(int n, int k, KeyFn key_
     }
 }
 
+// ------------------------------------------ keys held in registers
+//
+// The same k-th best key for a block whose threads hold the elements in
+// registers (the calibration kernel: thread t owns PER consecutive positions,
+// the first nv of them candidates).  Passes over all the keys read no memory,
+// so one histogram of kBins bins over the keys' own range is followed by
+// gathering the boundary bin, and its keys (at most kFew, else the range
+// narrows by another histogram) find their own rank: a thread counts the
+// gathered keys above and equal to its own, and the one whose ranks span k
+// publishes the result.  Five block barriers in the usual case.
+template <int T>
+struct SelectScratch {
+    // fewer keys need fewer bins, and one warp walks them all
+    static constexpr int kBins = T >= 512 ? 2048 : (T >= 256 ? 1024 : 512);
+    static constexpr int kFew = 256;  // keys that are ranked by counting
+    __align__(16) int bins[kBins];
+    __align__(16) uint32_t few[kFew];
+    uint32_t lo[32], hi[32];  // per-warp key ranges
+    int out[3];               // boundary bin, count above it left over, keys in it
+    uint32_t tau;
+    int need, eq;
+    int nfew;
+};
+
+// By one warp: the highest bin from which the count from the top reaches
+// `remaining`; out = {bin, how many of its keys are taken, its keys}.
+template <int BINS>
+__device__ __forceinline__ void boundary_bin(const int* bins, int remaining, int* out)
+{
+    constexpr int BL = BINS / 32;  // bins per lane
+    static_assert(BL == 64 || BL == 32 || BL == 16, "two, one or half a bin per lane below");
+    const int lane = threadIdx.x & 31;
+    const int4* b4 = reinterpret_cast<const int4*>(bins) + (BL / 4) * lane;
+    int mine = 0;
+#pragma unroll
+    for (int q = 0; q < BL / 4; ++q) {
+        const int4 v = b4[(q + lane) & (BL / 4 - 1)];
+        mine += v.x + v.y + v.z + v.w;
+    }
+    int incl = mine;  // keys in this lane's bins and above
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_down_sync(0xffffffffu, incl, o);
+        if (lane + o < 32) incl += y;
+    }
+    const uint32_t hit = __ballot_sync(0xffffffffu, incl >= remaining);
+    const int lb = hit ? 31 - __clz(hit) : 0;
+    const int above = __shfl_sync(0xffffffffu, incl - mine, lb);
+    // the boundary lane's bins: two, one or (below 32) at most one per lane
+    constexpr int PL = BL == 64 ? 2 : 1;
+    const int b0 = BL * lb + PL * lane;
+    const bool held = PL * lane < BL;
+    const int c0 = held ? bins[b0] : 0, c1 = (PL == 2) ? bins[b0 + 1] : 0;
+    const int pair = c0 + c1;
+    int inc2 = pair;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_down_sync(0xffffffffu, inc2, o);
+        if (lane + o < 32) inc2 += y;
+    }
+    const uint32_t hit2 = __ballot_sync(0xffffffffu, held && above + inc2 >= remaining);
+    const int l2 = hit2 ? 31 - __clz(hit2) : 0;
+    if (lane == l2) {
+        const int before = above + inc2 - pair;  // keys above this lane's bins
+        const bool top = PL == 2 && before + c1 >= remaining;
+        out[0] = top ? b0 + 1 : b0;
+        out[1] = (PL == 1 || top) ? remaining - before : remaining - before - c1;
+        out[2] = top ? c1 : c0;
+    }
+}
+
+// x: the thread's PER values, the first nv included (0 <= nv <= PER); 1 <= k
+// <= the block's included values; kmin / kmax: the thread's own key range.
+// Every thread returns the same result.  The scratch may be used again after
+// the call's last barrier: a second call's first writes touch only what no
+// thread reads after that barrier.
+template <int T, int PER>
+__device__ __forceinline__ SelectResult select_runs(const float* x, int nv, int k,
+                                                    SelectScratch<T>& sc, uint32_t kmin,
+                                                    uint32_t kmax)
+{
+    using S = SelectScratch<T>;
+    constexpr int kWarps = T / 32;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    kmin = __reduce_min_sync(0xffffffffu, kmin);
+    kmax = __reduce_max_sync(0xffffffffu, kmax);
+    if (lane == 0) {
+        sc.lo[warp] = kmin;
+        sc.hi[warp] = kmax;
+    }
+    if (threadIdx.x == 0) sc.nfew = 0;
+    for (int b = threadIdx.x; b < S::kBins / 4; b += T)
+        reinterpret_cast<int4*>(sc.bins)[b] = make_int4(0, 0, 0, 0);
+    __syncthreads();
+    uint32_t lo = __reduce_min_sync(0xffffffffu, lane < kWarps ? sc.lo[lane] : 0xffffffffu);
+    uint32_t last = __reduce_max_sync(0xffffffffu, lane < kWarps ? sc.hi[lane] : 0u) - lo;
+    // keys of the current range: [lo, lo + last]; bins of 2^shift keys
+    int shift = max(0, 32 - __clz(last | 1u) - (31 - __clz(S::kBins)));
+    int remaining = k;
+    while (true) {
+#pragma unroll
+        for (int q = 0; q < PER; ++q) {
+            const uint32_t d = float_key(x[q]) - lo;
+            if (q < nv && d <= last) atomicAdd(&sc.bins[d >> shift], 1);
+        }
+        __syncthreads();
+        if (warp == 0) boundary_bin<S::kBins>(sc.bins, remaining, sc.out);
+        __syncthreads();
+        lo += (uint32_t)sc.out[0] << shift;
+        remaining = sc.out[1];
+        const int in_bin = sc.out[2];
+        last = (1u << shift) - 1u;
+        if (shift == 0) return {lo, remaining, in_bin};
+        if (in_bin <= S::kFew) break;
+        // many keys in one bin (plateaus of equal scores): narrow the range
+        shift = max(0, shift - (31 - __clz(S::kBins)));
+        for (int b = threadIdx.x; b < S::kBins / 4; b += T)
+            reinterpret_cast<int4*>(sc.bins)[b] = make_int4(0, 0, 0, 0);
+        __syncthreads();
+    }
+    const int n = sc.out[2];
+#pragma unroll
+    for (int q = 0; q < PER; ++q) {
+        const uint32_t key = float_key(x[q]);
+        if (q < nv && key - lo <= last) sc.few[atomicAdd(&sc.nfew, 1)] = key;
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < n; i += T) {
+        const uint32_t key = sc.few[i];
+        int gt = 0, eq = 0;
+        for (int j = 0; j < n; ++j) {
+            const uint32_t o = sc.few[j];
+            gt += o > key;
+            eq += o == key;
+        }
+        if (gt < remaining && gt + eq >= remaining) {  // (equal keys write the same values)
+            sc.tau = key;
+            sc.need = remaining - gt;
+            sc.eq = eq;
+        }
+    }
+    __syncthreads();
+    return {sc.tau, sc.need, sc.eq};
+}
+
+// ------------------------------------------ keys behind an accessor
+
 template <typename KeyFn>
 __device__ SelectResult radix_select_by(int n, int k, KeyFn key_of, int* hist, int* bcast)
 {
