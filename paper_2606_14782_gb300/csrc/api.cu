@@ -91,6 +91,8 @@ struct bacon_ctx {
     float* lam = nullptr;
     float* lse2 = nullptr;
     float2* partial = nullptr;
+    uint8_t* taken = nullptr;  // adaptive head budgets: bitmap of the guaranteed candidates
+    uint2* key_range = nullptr;
     int* err = nullptr;
     int last_units = 0, last_N = 0;
     // staging buffers of bacon_compress_host
@@ -295,6 +297,7 @@ void free_ctx_buffers(bacon_ctx* c)
     c->ev_skipped.clear();
     c->ev_free.clear();
     void* bufs[] = {c->B,      c->Q,      c->E,      c->S,      c->V,      c->Bp,
+                    c->taken,  c->key_range,
                     c->lam,    c->lse2,   c->partial, c->err,   c->hq_buf, c->hk_buf,
                     c->hv_buf, c->hko_buf, c->hvo_buf, c->hidx_buf};
     for (void* b : bufs)
@@ -459,10 +462,19 @@ bacon_status compress_device(bacon_ctx* c, int R, const void* const* q, const vo
     a.do_select = adaptive ? 0 : 1;
     a.write_S = (c->p.keep_scores || adaptive) ? 1 : 0;
     a.err = c->err;
+    if (adaptive) {
+        a.taken = c->taken;
+        a.taken_stride = (N + 7) / 8;
+        a.guaranteed = guaranteed;
+        a.key_range = c->key_range;
+    }
     BACON_CUDA(launch_calibrate_select(s, calib_of(c), a, st), "calibrate_select launch");
     if (adaptive) {
         AdaptArgs ad;
         ad.S = S;
+        ad.taken = a.taken;
+        ad.taken_stride = a.taken_stride;
+        ad.key_range = a.key_range;
         ad.budget = layer_budget[0];
         ad.guaranteed = guaranteed;
         for (int i = 0; i < pairs; ++i) {
@@ -664,6 +676,8 @@ bacon_status bacon_init(bacon_ctx** out, int layers, int kv_heads, int q_heads, 
     if (e == cudaSuccess) e = dalloc(&c->lam, c->unit_cap);
     if (e == cudaSuccess) e = dalloc(&c->lse2, c->unit_cap * rows);
     if (e == cudaSuccess) e = dalloc(&c->partial, c->unit_cap * c->max_chunks * rows);
+    if (e == cudaSuccess) e = dalloc(&c->taken, c->unit_cap * (((size_t)prm.max_seq_len + 7) / 8));
+    if (e == cudaSuccess) e = dalloc(&c->key_range, c->unit_cap);
     if (e == cudaSuccess) e = dalloc(&c->err, 1);
     if (e == cudaSuccess) e = cudaMemset(c->err, 0, sizeof(int));
     if (e == cudaSuccess) e = dalloc(&c->d_maps, 2 * (size_t)kMaxPairs);
@@ -944,9 +958,9 @@ bacon_status bacon_compress_adaptive(bacon_ctx* ctx, int requests, const void* c
         if (!idx_out[i] || !aligned16(idx_out[i]))
             return fail(BACON_EINVAL, "index pointer of pair %d must be a 16-byte aligned device pointer", i);
     const int win = ctx->p.keep_window ? ctx->W : 0;
-    if (adaptive_smem(ctx->hkv, seq_len - win) > 200 * 1024)
-        return fail(BACON_EUNSUPPORTED, "kv_heads x candidates = %d exceeds the adaptive selection's %d",
-                    ctx->hkv * (seq_len - win), 200 * 1024);
+    if ((long long)ctx->hkv * (seq_len - win) > kMaxAdaptive)
+        return fail(BACON_EUNSUPPORTED, "kv_heads x candidates = %lld exceeds the adaptive selection's %d",
+                    (long long)ctx->hkv * (seq_len - win), kMaxAdaptive);
     const int kept = budget < seq_len ? budget : seq_len;
     const int guaranteed = (int)floor((double)alpha * (double)(kept - win));
     DeviceGuard dg(ctx->device);

@@ -74,60 +74,12 @@ __device__ __forceinline__ void block_sums(float (&v)[NV], float* red)
         for (int i = 0; i < NV; ++i) v[i] += __shfl_xor_sync(0xffffffffu, v[i], o);
 }
 
-// Exclusive prefix sum of one int per thread, in thread order; total receives
-// the sum.  One block barrier: every warp scans the warps' sums itself.
-// warp_sums holds 32 ints and is not used again before the next barrier.
-template <int T>
-__device__ __forceinline__ int block_exclusive_scan(int v, int* warp_sums, int& total)
-{
-    constexpr int kWarps = T / 32;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    int incl = v;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const int y = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += y;
-    }
-    if (lane == 31) warp_sums[warp] = incl;
-    __syncthreads();
-    const int w = lane < kWarps ? warp_sums[lane] : 0;
-    int wi = w;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const int y = __shfl_up_sync(0xffffffffu, wi, o);
-        if (lane >= o) wi += y;
-    }
-    total = __shfl_sync(0xffffffffu, wi, 31);
-    return __shfl_sync(0xffffffffu, wi - w, warp) + incl - v;
-}
-
 // Ask L2 to fetch the n floats at p (one prefetch per 128-byte line, every
 // address inside the array), so that later loads of them hit L2.
 __device__ __forceinline__ void prefetch_l2(const float* p, int n)
 {
     for (int i = (int)threadIdx.x * 32; i < n; i += (int)blockDim.x * 32)
         asm volatile("prefetch.global.L2 [%0];" ::"l"(p + i));
-}
-
-// x[k] = src[i0 + k] for the thread's PER positions (0 at and past n), with
-// 16-byte loads when the run is whole and aligned (n % 4 == 0).
-template <int PER>
-__device__ __forceinline__ void load_run(const float* __restrict__ src, int i0, int n, float* x)
-{
-    if ((n & 3) == 0 && i0 + PER <= n) {
-        const float4* s4 = reinterpret_cast<const float4*>(src + i0);
-#pragma unroll
-        for (int q = 0; q < PER / 4; ++q) {
-            const float4 v = __ldg(s4 + q);
-            x[4 * q] = v.x;
-            x[4 * q + 1] = v.y;
-            x[4 * q + 2] = v.z;
-            x[4 * q + 3] = v.w;
-        }
-    } else {
-#pragma unroll
-        for (int k = 0; k < PER; ++k) x[k] = i0 + k < n ? src[i0 + k] : 0.f;
-    }
 }
 
 // dst[i0 + k] = x[k] for the positions below n.
@@ -397,7 +349,9 @@ __device__ __forceinline__ void pool_run(const float* __restrict__ Bu, int i0, i
 // score: the keys of the two selections) stays in registers, and so does V
 // where a run is 8 positions; longer runs form V after the first selection,
 // with the backbone parked in the thread's own column of shared memory.
-template <int T, int PER>
+// ADAPT: the head's guaranteed share and its key range for the adaptive
+// selection take the place of Eq. 17.
+template <int T, int PER, bool ADAPT>
 __device__ __forceinline__ void calibrate_unit(const Shape& s, const Calib& c, const CalibArgs& a,
                                                int u, float* lam_out, int32_t* idx_pair)
 {
@@ -517,6 +471,37 @@ __device__ __forceinline__ void calibrate_unit(const Shape& s, const Calib& c, c
         }
     }
 
+    if constexpr (ADAPT) {
+        // adaptive head budgets: the head's own best candidates as a bitmap of
+        // positions, and the key range of its scores
+        const int sure = min(a.guaranteed, keep);
+        uint32_t mem = 0u;
+        if (keep >= n_cand) {
+            mem = (1u << nv) - 1u;
+        } else if (sure > 0) {
+            const SelectResult sel = select_runs<T, PER>(b, nv, sure, sel_sm, skmin, skmax);
+            mem = members<PER>(b, nv, sel, ties_before<T, PER>(b, nv, sel, ties[1]));
+        }
+        uint8_t* map = a.taken + (size_t)u * a.taken_stride;
+#pragma unroll
+        for (int q = 0; q < PER / 8; ++q)
+            if (i0 + 8 * q < n_cand) map[i0 / 8 + q] = (uint8_t)(mem >> (8 * q));
+        __shared__ uint32_t ranges[2][32];
+        const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+        skmin = __reduce_min_sync(0xffffffffu, skmin);
+        skmax = __reduce_max_sync(0xffffffffu, skmax);
+        if (lane == 0) {
+            ranges[0][warp] = skmin;
+            ranges[1][warp] = skmax;
+        }
+        __syncthreads();
+        if (warp == 0) {
+            skmin = __reduce_min_sync(0xffffffffu, lane < T / 32 ? ranges[0][lane] : 0xffffffffu);
+            skmax = __reduce_max_sync(0xffffffffu, lane < T / 32 ? ranges[1][lane] : 0u);
+            if (lane == 0) a.key_range[u] = make_uint2(skmin, skmax);
+        }
+        return;
+    }
     if (!a.do_select) return;
     // ---- Eq. 17: the K best candidates by S, ascending, then the window
     int32_t* out = idx_pair + (size_t)h * kept_total;
@@ -535,12 +520,12 @@ __device__ __forceinline__ void calibrate_unit(const Shape& s, const Calib& c, c
     for (int w = threadIdx.x; w < win; w += T) out[keep + w] = N - W + w;
 }
 
-template <int T, int PER>
+template <int T, int PER, bool ADAPT>
 __global__ void __launch_bounds__(T, 1024 / T)
 calibrate_select_kernel(Shape s, Calib c, CalibArgs a)
 {
     const int u = blockIdx.x;
-    calibrate_unit<T, PER>(s, c, a, u, a.lambda + u, a.idx[u / s.hkv]);
+    calibrate_unit<T, PER, ADAPT>(s, c, a, u, a.lambda + u, a.idx[u / s.hkv]);
 }
 
 // Several hyper-parameter sets over the same B and residuals: CTA (u, v)
@@ -553,7 +538,7 @@ calibrate_sweep_kernel(Shape s, CalibTable t, CalibArgs a)
 {
     const int u = blockIdx.x, v = blockIdx.y;
     float* lam = a.lambda ? a.lambda + (size_t)v * s.units + u : nullptr;
-    calibrate_unit<T, PER>(s, t.c[v], a, u, lam,
+    calibrate_unit<T, PER, false>(s, t.c[v], a, u, lam,
                            a.idx[u / s.hkv] + (size_t)v * a.idx_variant_stride);
 }
 
@@ -563,14 +548,14 @@ constexpr size_t smem_bytes()
     return PER > 8 ? (size_t)T * PER * sizeof(float) : 0;
 }
 
-template <int T, int PER>
+template <int T, int PER, bool ADAPT>
 cudaError_t launch_select_t(const Shape& s, const Calib& c, const CalibArgs& a, cudaStream_t st)
 {
     constexpr size_t sm = smem_bytes<T, PER>();
-    cudaError_t e = cudaFuncSetAttribute(calibrate_select_kernel<T, PER>,
+    cudaError_t e = cudaFuncSetAttribute(calibrate_select_kernel<T, PER, ADAPT>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
-    calibrate_select_kernel<T, PER><<<s.units, T, sm, st>>>(s, c, a);
+    calibrate_select_kernel<T, PER, ADAPT><<<s.units, T, sm, st>>>(s, c, a);
     return cudaGetLastError();
 }
 
@@ -605,7 +590,11 @@ struct SelectLaunch {
     const CalibArgs& a;
     cudaStream_t st;
     template <int T, int PER>
-    cudaError_t run() const { return launch_select_t<T, PER>(s, c, a, st); }
+    cudaError_t run() const
+    {
+        return a.taken ? launch_select_t<T, PER, true>(s, c, a, st)
+                       : launch_select_t<T, PER, false>(s, c, a, st);
+    }
 };
 
 struct SweepLaunch {

@@ -94,6 +94,13 @@ struct CalibArgs {
     int budget[kMaxPairs];       // kept tokens per head (window included)
     int calib_budget[kMaxPairs]; // budget that sets K in Eq. 12
     long long idx_variant_stride = 0;  // sweep only: elements between variants' indices
+    // adaptive head budgets (taken null otherwise; do_select is 0 then): each
+    // unit's `guaranteed` best candidates as a bitmap of positions,
+    // taken_stride bytes per unit, and the range of its candidates' keys
+    uint8_t* taken = nullptr;
+    int taken_stride = 0;
+    int guaranteed = 0;
+    uint2* key_range = nullptr;
     int compute_scores;  // 1: V, B~, lambda, S from B and the residuals
     int do_select;       // 1: top-B selection into idx
     int write_S;
@@ -112,9 +119,13 @@ struct CalibTable {
 cudaError_t launch_calibrate_sweep(const Shape& s, const CalibTable& t, int variants,
                                    const CalibArgs& a, cudaStream_t st);
 
-// AdaKV-style selection over the heads of each (request, layer).
+// AdaKV-style selection over the heads of each (request, layer), after the
+// calibration has marked each head's guaranteed candidates.
 struct AdaptArgs {
     const float* S;              // [units][N] final scores (0 off-candidates)
+    const uint8_t* taken;        // CalibArgs' bitmap, taken_stride bytes per unit
+    int taken_stride;
+    const uint2* key_range;      // [units]
     int budget;                  // average per-head budget (window included)
     int guaranteed;              // g = floor(alpha K) candidates per head first
     int32_t* idx[kMaxPairs];     // per pair: flat [Hkv * kept] positions, heads in order
@@ -123,8 +134,9 @@ struct AdaptArgs {
 };
 cudaError_t launch_adaptive_select(const Shape& s, int keep_window, const AdaptArgs& a,
                                    cudaStream_t st);
-// Dynamic shared memory of the adaptive selection (one byte per candidate).
-size_t adaptive_smem(int kv_heads, int n_cand);
+// Most candidates of one (request, layer), over its kv-heads, that the
+// adaptive selection takes.
+constexpr int kMaxAdaptive = 200 * 1024;
 // Gather into the flat per-layer layout of the adaptive selection.
 cudaError_t launch_gather_flat(const GatherTable& tab, const Shape& s, const int32_t* counts,
                                int* err, cudaStream_t st);

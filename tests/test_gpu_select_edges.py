@@ -55,3 +55,57 @@ def test_selections_match_a_stable_sort(n, distinct):
         floor = 1e-6 * Bp.double().gather(-1, top).amax(-1) / (sv + 1e-8)
         assert ((lam.double() - ref).abs() <= 2e-4 * ref + floor).all(), (keep, lam, ref)
         ctx.close()
+
+
+def _adaptive_reference(S, keep, sure):
+    """Membership [H, ncand] of one layer: each head's own best, then the best
+    of the rest jointly (ties to the lower head, then the lower position)."""
+    h, ncand = S.shape
+    taken = torch.zeros_like(S, dtype=torch.bool)
+    if keep >= ncand:
+        return ~taken
+    if sure:
+        taken.scatter_(1, _best(S, sure), True)
+    rest = h * (keep - sure)
+    if rest:
+        free = (~taken).view(-1).nonzero()[:, 0]
+        taken.view(-1)[free[_best(S.reshape(-1)[free], rest)]] = True
+    return taken
+
+
+@pytest.mark.parametrize("distinct", [1, 5, 0])
+@pytest.mark.parametrize("n,h,win", [
+    (12, 3, 8), (300, 1, 8), (1024, 32, 8), (1027, 5, 8), (2500, 4, 8), (8193, 3, 8),
+    (16384, 4, 8), (16390, 2, 8), (1027, 5, 0),
+])
+def test_adaptive_matches_a_stable_sort(n, h, win, distinct):
+    g = torch.Generator(device="cuda").manual_seed(77 * distinct + n)
+    layers, d, w = 2, 64, 8
+    q = torch.randn(1, layers, h, w, d, generator=g, device="cuda").bfloat16()
+    k = torch.randn(1, layers, h, n, d, generator=g, device="cuda")
+    if distinct:
+        pick = torch.randint(0, distinct, (n,), generator=g, device="cuda")
+        k = k[..., :1, :].expand_as(k) if distinct == 1 else k[..., pick % n, :]
+    k = k.bfloat16().contiguous()
+    ncand = n - win
+    for budget in sorted({w, w + 4, min(n, (w + n // 12) // 4 * 4), n // 4 * 4, n - 1, n}):
+        if budget < w or h * budget % 4:  # the binding's index blocks are 16-byte aligned
+            continue
+        ctx = bacon.Context(layers, h, h, d, w, 7, budget, max_seq_len=n, max_requests=1,
+                            keep_window=int(win > 0))
+        for alpha in (0.0, 0.2, 1.0):
+            ko, vo, idx, counts = ctx.compress_adaptive(q, k, k, budget, alpha)
+            S = ctx.scores("S").view(layers, h, n)[..., :ncand]
+            ctx.sync()
+            keep = budget - win
+            sure = int(alpha * keep) if alpha in (0.0, 1.0) else int(
+                torch.tensor(alpha, dtype=torch.float32).double().item() * keep)
+            for l in range(layers):
+                m = _adaptive_reference(S[l], keep, sure)
+                tail = torch.arange(ncand, n, device="cuda")
+                want = torch.cat([torch.cat([x.nonzero()[:, 0], tail]) for x in m])
+                assert torch.equal(idx[0, l].long(), want), (budget, alpha, l)
+                assert torch.equal(counts[0, l].long(), m.sum(1) + win), (budget, alpha, l)
+                heads = torch.repeat_interleave(torch.arange(h, device="cuda"), counts[0, l].long())
+                assert torch.equal(ko[0, l], k[0, l][heads, want])
+        ctx.close()
