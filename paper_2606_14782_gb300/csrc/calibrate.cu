@@ -460,6 +460,7 @@ __device__ __forceinline__ void calibrate_unit(const Shape& s, const Calib& c, c
             }
         }
         if (a.write_S) store_run<PER>(a.S + (size_t)u * N, i0, N, b);
+        if (a.S_copy) store_run<PER>(a.S_copy + (size_t)u * N, i0, N, b);
     } else {
         load_run<PER>(a.S + (size_t)u * N, i0, N, b);
 #pragma unroll

@@ -87,6 +87,7 @@ struct CalibArgs {
     long long ring_req_stride;
     int layer0;
     float* S;            // [units][N] final score (written when write_S)
+    float* S_copy = nullptr;  // optional [units][N], 16-byte aligned: S once more
     float* V;            // optional [units][N]
     float* Bp;           // optional [units][N]
     float* lambda;       // [units]

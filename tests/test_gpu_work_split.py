@@ -59,3 +59,24 @@ def test_few_units_and_many_give_the_same_bits(group, window, head_dim, seq_len)
     assert torch.equal(B, whole["B"][1, 2]) and torch.equal(Q, whole["Q"][1, 2])
     st.close()
     ctx.close()
+
+
+@pytest.mark.parametrize("offset", [0, 1, 2, 4])
+def test_scores_out_at_any_float_alignment(offset):
+    """Aligned score rows are stored by the kernel, others copied: same bits."""
+    hkv, n, w = 2, 1156, 32
+    wl = workloads.CONFIGS["tiny"].with_(layers=1, q_heads=8, kv_heads=hkv, head_dim=64, seq_len=n,
+                                         visual=(16, 1000))
+    x = workloads.generate(wl, seed=3, device="cuda")
+    ctx = bacon.Context(1, hkv, 8, 64, w, 7, 100, max_seq_len=n, max_requests=1)
+    st = bacon.State(ctx)
+    want = st.score_layer(0, x.qwin[0, 0], x.k[0, 0], scores_out=True)
+    buf = torch.full((hkv * n + 8,), 7.0, device="cuda")
+    st.reset()
+    st.score_layer(0, x.qwin[0, 0], x.k[0, 0],
+                   scores_out=buf[offset:offset + hkv * n].view(hkv, n))
+    ctx.sync()
+    assert torch.equal(buf[offset:offset + hkv * n].view(hkv, n), want)
+    assert (buf[:offset] == 7.0).all() and (buf[offset + hkv * n:] == 7.0).all()
+    st.close()
+    ctx.close()
