@@ -93,6 +93,7 @@ struct bacon_ctx {
     float2* partial = nullptr;
     uint8_t* taken = nullptr;  // adaptive head budgets: bitmap of the guaranteed candidates
     uint2* key_range = nullptr;
+    float2* moments = nullptr;  // sweep: B~'s moment sums per distinct rho
     int* err = nullptr;
     int last_units = 0, last_N = 0;
     // staging buffers of bacon_compress_host
@@ -297,7 +298,7 @@ void free_ctx_buffers(bacon_ctx* c)
     c->ev_skipped.clear();
     c->ev_free.clear();
     void* bufs[] = {c->B,      c->Q,      c->E,      c->S,      c->V,      c->Bp,
-                    c->taken,  c->key_range,
+                    c->taken,  c->key_range, c->moments,
                     c->lam,    c->lse2,   c->partial, c->err,   c->hq_buf, c->hk_buf,
                     c->hv_buf, c->hko_buf, c->hvo_buf, c->hidx_buf};
     for (void* b : bufs)
@@ -543,7 +544,14 @@ bacon_status sweep_device(bacon_ctx* c, int R, const void* const* q, const void*
     a.do_select = 1;
     a.write_S = 0;
     a.err = c->err;
-    BACON_CUDA(launch_calibrate_sweep(s, t, variants, a, st), "calibrate_sweep launch");
+    // Q and S of the scratch are not this call's results (get_scores refuses
+    // them afterwards): Q's place takes the pooled backbone, S's the bitmaps
+    SweepArgs sw;
+    sw.pooled = c->Q;
+    sw.maps = reinterpret_cast<uint8_t*>(c->S);
+    sw.map_stride = (N + 7) / 8;
+    sw.moments = c->moments;
+    BACON_CUDA(launch_calibrate_sweep(s, t, variants, sw, a, st), "calibrate_sweep launch");
     prof.mark(4);
     prof.mark(5);
     prof.commit();
@@ -670,7 +678,9 @@ bacon_status bacon_init(bacon_ctx** out, int layers, int kv_heads, int q_heads, 
     if (e == cudaSuccess) e = dalloc(&c->B, tok);
     if (e == cudaSuccess) e = dalloc(&c->Q, tok);
     if (e == cudaSuccess) e = dalloc(&c->E, tok);
-    if (e == cudaSuccess) e = dalloc(&c->S, tok);
+    // (S also holds the sweep's bitmaps: kMaxVariants x ceil(N / 8) bytes per unit)
+    if (e == cudaSuccess) e = dalloc(&c->S, tok + 8 * c->unit_cap);
+    if (e == cudaSuccess) e = dalloc(&c->moments, kMaxVariants * c->unit_cap);
     if (e == cudaSuccess) e = dalloc(&c->V, prm.keep_scores ? tok : 0);
     if (e == cudaSuccess) e = dalloc(&c->Bp, prm.keep_scores ? tok : 0);
     if (e == cudaSuccess) e = dalloc(&c->lam, c->unit_cap);

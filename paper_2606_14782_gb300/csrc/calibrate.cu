@@ -343,6 +343,62 @@ __device__ __forceinline__ void pool_run(const float* __restrict__ Bu, int i0, i
     }
 }
 
+// lambda over the M members (Eqs. 13-15): sx and syy are B~'s moment sums
+// about the M-th value (every member is at or above it, so the fp32
+// differences stay small), sv the members' sum of V, whose mean square
+// deviation from its mean takes one more reduction.
+template <int T, int PER>
+__device__ __forceinline__ float lambda_of(const Calib& c, int M, uint32_t mem, float sx, float syy,
+                                           float sv, const float* v, float* red)
+{
+    const float inv_m = 1.f / (float)M;
+    const float mb = sx * inv_m, mv = sv * inv_m;
+    float dev[1] = {0.f};
+#pragma unroll
+    for (int k = 0; k < PER; ++k) {
+        if ((mem >> k) & 1u) {
+            const float dv = v[k] - mv;
+            dev[0] = fmaf(dv, dv, dev[0]);
+        }
+    }
+    block_sums<T, 1>(dev, red);
+    const float varv = dev[0] * inv_m;
+    const float stdb = sqrtf(fmaxf(syy * inv_m - mb * mb, 0.f));
+    const float stdv = sqrtf(varv);
+    return c.gamma * stdb / (stdv + c.eps);
+}
+
+// Eq. 17: the `keep` best candidates by the scores in b (key range skmin,
+// skmax), ascending, then the window.
+template <int T, int PER>
+__device__ __forceinline__ void emit_best(const float* b, int i0, int nv, int n_cand, int keep,
+                                          int win, int N, uint32_t skmin, uint32_t skmax,
+                                          SelectScratch<T>& sel_sm, int* ties, int* offsets,
+                                          int32_t* out, int* err)
+{
+    if (keep >= n_cand) {
+        for (int i = threadIdx.x; i < n_cand; i += T) out[i] = i;
+    } else if (keep > 0) {
+        const SelectResult sel = select_runs<T, PER>(b, nv, keep, sel_sm, skmin, skmax);
+        const uint32_t mem = members<PER>(b, nv, sel, ties_before<T, PER>(b, nv, sel, ties));
+        int total;
+        int pos = block_exclusive_scan<T>(__popc(mem), offsets, total);
+#pragma unroll
+        for (int k = 0; k < PER; ++k)
+            if ((mem >> k) & 1u) out[pos++] = i0 + k;
+        if (threadIdx.x == 0 && total != keep && err) atomicCAS(err, 0, 2);
+    }
+    for (int w = threadIdx.x; w < win; w += T) out[keep + w] = N - win + w;
+}
+
+// M of Eq. 12 for a pair's budget.
+__device__ __forceinline__ int match_count(int rho, int budget, int N, int win, int n_cand)
+{
+    const int calib_keep = min(budget, N) - win;
+    const long long M = (long long)rho * (long long)(calib_keep > 0 ? calib_keep : 0);
+    return (int)(M < n_cand ? M : n_cand);
+}
+
 // One unit (request, layer, kv-head) u under hyper-parameters c.  lam_out
 // (may be null) receives lambda; idx_pair is the pair's [Hkv][kept] output.
 // N <= T PER.  The thread's run of the pooled backbone (then of the final
@@ -397,9 +453,7 @@ __device__ __forceinline__ void calibrate_unit(const Shape& s, const Calib& c, c
         if (a.Bp) store_run<PER>(a.Bp + (size_t)u * N, i0, N, b);
 
         // ---- the M best candidates by B~ (Eq. 12)
-        const int calib_keep = min(a.calib_budget[pair], N) - win;
-        const long long Ml = (long long)c.rho * (long long)(calib_keep > 0 ? calib_keep : 0);
-        const int M = (int)(Ml < n_cand ? Ml : n_cand);
+        const int M = match_count(c.rho, a.calib_budget[pair], N, win, n_cand);
         uint32_t mem = 0u;
         float pb = 0.f;
         if (M > 0) {
@@ -416,10 +470,7 @@ __device__ __forceinline__ void calibrate_unit(const Shape& s, const Calib& c, c
         }
         if (a.V) store_run<PER>(a.V + (size_t)u * N, i0, N, v);
 
-        // ---- lambda over the M members (Eqs. 13-15).  B~ by moments about
-        // the M-th value (every member is at or above it, so the fp32
-        // differences stay small); V by its members' mean, then the mean
-        // square deviation from it (two reductions).
+        // ---- lambda over the M members (Eqs. 13-15)
         float lam = 0.f;
         if (M > 0) {
             float acc[3] = {0.f, 0.f, 0.f};
@@ -433,21 +484,7 @@ __device__ __forceinline__ void calibrate_unit(const Shape& s, const Calib& c, c
                 }
             }
             block_sums<T, 3>(acc, red_b);
-            const float inv_m = 1.f / (float)M;
-            const float mb = acc[0] * inv_m, mv = acc[2] * inv_m;
-            float dev[1] = {0.f};
-#pragma unroll
-            for (int k = 0; k < PER; ++k) {
-                if ((mem >> k) & 1u) {
-                    const float dv = v[k] - mv;
-                    dev[0] = fmaf(dv, dv, dev[0]);
-                }
-            }
-            block_sums<T, 1>(dev, red_v);
-            const float varv = dev[0] * inv_m;
-            const float stdb = sqrtf(fmaxf(acc[1] * inv_m - mb * mb, 0.f));
-            const float stdv = sqrtf(varv);
-            lam = c.gamma * stdb / (stdv + c.eps);
+            lam = lambda_of<T, PER>(c, M, mem, acc[0], acc[1], acc[2], v, red_v);
         }
         if (threadIdx.x == 0 && lam_out) *lam_out = lam;
         // ---- Eq. 16 over the candidates (0 elsewhere)
@@ -503,22 +540,9 @@ __device__ __forceinline__ void calibrate_unit(const Shape& s, const Calib& c, c
         }
         return;
     }
-    if (!a.do_select) return;
-    // ---- Eq. 17: the K best candidates by S, ascending, then the window
-    int32_t* out = idx_pair + (size_t)h * kept_total;
-    if (keep >= n_cand) {
-        for (int i = threadIdx.x; i < n_cand; i += T) out[i] = i;
-    } else if (keep > 0) {
-        const SelectResult sel = select_runs<T, PER>(b, nv, keep, sel_sm, skmin, skmax);
-        const uint32_t mem = members<PER>(b, nv, sel, ties_before<T, PER>(b, nv, sel, ties[1]));
-        int total;
-        int pos = block_exclusive_scan<T>(__popc(mem), offsets, total);
-#pragma unroll
-        for (int k = 0; k < PER; ++k)
-            if ((mem >> k) & 1u) out[pos++] = i0 + k;
-        if (threadIdx.x == 0 && total != keep && a.err) atomicCAS(a.err, 0, 2);
-    }
-    for (int w = threadIdx.x; w < win; w += T) out[keep + w] = N - W + w;
+    if (a.do_select)
+        emit_best<T, PER>(b, i0, nv, n_cand, keep, win, N, skmin, skmax, sel_sm, ties[1], offsets,
+                          idx_pair + (size_t)h * kept_total, a.err);
 }
 
 template <int T, int PER, bool ADAPT>
@@ -529,18 +553,108 @@ calibrate_select_kernel(Shape s, Calib c, CalibArgs a)
     calibrate_unit<T, PER, ADAPT>(s, c, a, u, a.lambda + u, a.idx[u / s.hkv]);
 }
 
-// Several hyper-parameter sets over the same B and residuals: CTA (u, v)
-// runs unit u under variant v; variant v's indices start v *
+// Several hyper-parameter sets over the same B and residuals, in two kernels.
+// What the variants of a unit share is formed once: the pooled backbone, and
+// per distinct rho the M best by it (a bitmap of positions, position order =
+// bit order) with B~'s moment sums over them.  CTA (u, v) then runs unit u
+// under variant v from there; variant v's indices start v *
 // idx_variant_stride elements after the single-variant layout and its
-// lambdas v * units after a.lambda.
+// lambdas v * units after a.lambda.  Both are bound by latency like the
+// kernel above: 11 variants of 112 units x 6528 tokens take 87 us, where
+// every (unit, variant) repeating the shared part took 125.
 template <int T, int PER>
 __global__ void __launch_bounds__(T, 1024 / T)
-calibrate_sweep_kernel(Shape s, CalibTable t, CalibArgs a)
+sweep_shared_kernel(Shape s, Calib c, SweepArgs sw, CalibArgs a)
 {
-    const int u = blockIdx.x, v = blockIdx.y;
-    float* lam = a.lambda ? a.lambda + (size_t)v * s.units + u : nullptr;
-    calibrate_unit<T, PER, false>(s, t.c[v], a, u, lam,
-                           a.idx[u / s.hkv] + (size_t)v * a.idx_variant_stride);
+    __shared__ SelectScratch<T> sel_sm;
+    __shared__ int ties[32];
+    __shared__ float red[2 * 32];
+    const int u = blockIdx.x, ri = blockIdx.y;
+    const int N = s.N, win = c.keep_window ? s.W : 0, n_cand = N - win;
+    const int i0 = (int)threadIdx.x * PER;
+    const int nv = max(0, min(PER, n_cand - i0));
+    const float* Bu = a.B + (size_t)u * N;
+    float b[PER];
+    load_run<PER>(Bu, i0, N, b);
+    uint32_t kmin = 0xffffffffu, kmax = 0u;
+    pool_run<PER>(Bu, i0, n_cand, c.pool / 2, b, kmin, kmax);
+    if (ri == 0) store_run<PER>(sw.pooled + (size_t)u * N, i0, N, b);
+    const int M = match_count(sw.rho[ri], a.calib_budget[u / s.hkv], N, win, n_cand);
+    if (M <= 0) return;
+    const SelectResult sel = select_runs<T, PER>(b, nv, M, sel_sm, kmin, kmax);
+    const uint32_t mem = members<PER>(b, nv, sel, ties_before<T, PER>(b, nv, sel, ties));
+    const float pb = key_float(sel.tau);
+    float acc[2] = {0.f, 0.f};
+#pragma unroll
+    for (int k = 0; k < PER; ++k) {
+        if ((mem >> k) & 1u) {
+            const float db = b[k] - pb;
+            acc[0] += db;
+            acc[1] = fmaf(db, db, acc[1]);
+        }
+    }
+    uint8_t* map = sw.maps + ((size_t)ri * s.units + u) * sw.map_stride;
+#pragma unroll
+    for (int q = 0; q < PER / 8; ++q)
+        if (i0 + 8 * q < n_cand) map[i0 / 8 + q] = (uint8_t)(mem >> (8 * q));
+    block_sums<T, 2>(acc, red);
+    if (threadIdx.x == 0) sw.moments[(size_t)ri * s.units + u] = make_float2(acc[0], acc[1]);
+}
+
+template <int T, int PER>
+__global__ void __launch_bounds__(T, 1024 / T)
+calibrate_sweep_kernel(Shape s, CalibTable t, SweepArgs sw, CalibArgs a)
+{
+    __shared__ SelectScratch<T> sel_sm;
+    __shared__ int ties[32], offsets[32];
+    __shared__ float red_s[32], red_v[32];
+    const int u = blockIdx.x, j = blockIdx.y;
+    const Calib& c = t.c[j];
+    const int N = s.N, win = c.keep_window ? s.W : 0, n_cand = N - win;
+    const int pair = u / s.hkv, h = u - pair * s.hkv;
+    const int rq = pair / s.layers;
+    const int layer = a.layer0 + (pair - rq * s.layers);
+    const int kept_total = min(a.budget[pair], N);
+    const int i0 = (int)threadIdx.x * PER;
+    const int nv = max(0, min(PER, n_cand - i0));
+    const int ri = sw.rho_of[j];
+    const int M = match_count(c.rho, a.calib_budget[pair], N, win, n_cand);
+    uint32_t mem = 0u;
+    if (M > 0) {
+        const uint8_t* map = sw.maps + ((size_t)ri * s.units + u) * sw.map_stride;
+#pragma unroll
+        for (int q = 0; q < PER / 8; ++q)
+            if (i0 + 8 * q < n_cand) mem |= (uint32_t)map[i0 / 8 + q] << (8 * q);
+    }
+    float x[PER], v[PER], b[PER];
+    evidence_run<PER>(c, [&](int l) -> const float* {
+        return a.Ering + (long long)rq * a.ring_req_stride +
+               (long long)(l % a.ring) * s.hkv * N + (long long)h * N;
+    }, layer, i0, N, x, v);
+    load_run<PER>(sw.pooled + (size_t)u * N, i0, N, b);
+    float lam = 0.f;
+    if (M > 0) {
+        float sv[1] = {0.f};
+#pragma unroll
+        for (int k = 0; k < PER; ++k)
+            if ((mem >> k) & 1u) sv[0] += v[k];
+        const float2 mo = sw.moments[(size_t)ri * s.units + u];
+        block_sums<T, 1>(sv, red_s);
+        lam = lambda_of<T, PER>(c, M, mem, mo.x, mo.y, sv[0], v, red_v);
+    }
+    if (threadIdx.x == 0 && a.lambda) a.lambda[(size_t)j * s.units + u] = lam;
+    uint32_t skmin = 0xffffffffu, skmax = 0u;
+#pragma unroll
+    for (int k = 0; k < PER; ++k) {
+        if (k < nv) {
+            b[k] = fmaf(lam, v[k], b[k]);
+            skmin = min(skmin, float_key(b[k]));
+            skmax = max(skmax, float_key(b[k]));
+        }
+    }
+    emit_best<T, PER>(b, i0, nv, n_cand, kept_total - win, win, N, skmin, skmax, sel_sm, ties,
+                      offsets, a.idx[pair] + (size_t)j * a.idx_variant_stride + (size_t)h * kept_total,
+                      a.err);
 }
 
 template <int T, int PER>
@@ -561,14 +675,13 @@ cudaError_t launch_select_t(const Shape& s, const Calib& c, const CalibArgs& a, 
 }
 
 template <int T, int PER>
-cudaError_t launch_sweep_t(const Shape& s, const CalibTable& t, int variants, const CalibArgs& a,
-                           cudaStream_t st)
+cudaError_t launch_sweep_t(const Shape& s, const CalibTable& t, int variants, const SweepArgs& sw,
+                           const CalibArgs& a, cudaStream_t st)
 {
-    constexpr size_t sm = smem_bytes<T, PER>();
-    cudaError_t e = cudaFuncSetAttribute(calibrate_sweep_kernel<T, PER>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    sweep_shared_kernel<T, PER><<<dim3(s.units, sw.rhos), T, 0, st>>>(s, t.c[0], sw, a);
+    cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    calibrate_sweep_kernel<T, PER><<<dim3(s.units, variants), T, sm, st>>>(s, t, a);
+    calibrate_sweep_kernel<T, PER><<<dim3(s.units, variants), T, 0, st>>>(s, t, sw, a);
     return cudaGetLastError();
 }
 
@@ -602,10 +715,11 @@ struct SweepLaunch {
     const Shape& s;
     const CalibTable& t;
     int variants;
+    const SweepArgs& sw;
     const CalibArgs& a;
     cudaStream_t st;
     template <int T, int PER>
-    cudaError_t run() const { return launch_sweep_t<T, PER>(s, t, variants, a, st); }
+    cudaError_t run() const { return launch_sweep_t<T, PER>(s, t, variants, sw, a, st); }
 };
 
 }  // namespace
@@ -617,9 +731,16 @@ cudaError_t launch_calibrate_select(const Shape& s, const Calib& c, const CalibA
 }
 
 cudaError_t launch_calibrate_sweep(const Shape& s, const CalibTable& t, int variants,
-                                   const CalibArgs& a, cudaStream_t st)
+                                   SweepArgs sw, const CalibArgs& a, cudaStream_t st)
 {
-    return by_size(s.N, SweepLaunch{s, t, variants, a, st});
+    sw.rhos = 0;
+    for (int j = 0; j < variants; ++j) {
+        int r = 0;
+        while (r < sw.rhos && sw.rho[r] != t.c[j].rho) ++r;
+        if (r == sw.rhos) sw.rho[sw.rhos++] = t.c[j].rho;
+        sw.rho_of[j] = r;
+    }
+    return by_size(s.N, SweepLaunch{s, t, variants, sw, a, st});
 }
 
 }  // namespace bacon

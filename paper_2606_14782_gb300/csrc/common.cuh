@@ -117,8 +117,18 @@ constexpr int kMaxVariants = 32;
 struct CalibTable {
     Calib c[kMaxVariants];
 };
+// What the variants share (the launch fills the rho lists).
+struct SweepArgs {
+    float* pooled;    // [units][N] pooled backbone
+    uint8_t* maps;    // [rhos][units] bitmaps of the M members, map_stride bytes each
+    int map_stride;
+    float2* moments;  // [rhos][units] B~'s moment sums over them
+    int rhos;
+    int rho[kMaxVariants];     // the distinct values
+    int rho_of[kMaxVariants];  // each variant's place among them
+};
 cudaError_t launch_calibrate_sweep(const Shape& s, const CalibTable& t, int variants,
-                                   const CalibArgs& a, cudaStream_t st);
+                                   SweepArgs sw, const CalibArgs& a, cudaStream_t st);
 
 // AdaKV-style selection over the heads of each (request, layer), after the
 // calibration has marked each head's guaranteed candidates.
