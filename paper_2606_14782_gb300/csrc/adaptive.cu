@@ -36,6 +36,7 @@ adaptive_select_kernel(Shape s, int keep_window, AdaptArgs a)
     __shared__ SelectScratch<kThreads> sel_sm;
     __shared__ int ties[32], offsets[32];
 
+    after_previous();
     const int pair = blockIdx.x;
     const int H = s.hkv, N = s.N, W = s.W;
     const int win = keep_window ? W : 0;
@@ -143,6 +144,7 @@ __global__ void __launch_bounds__(256)
 gather_flat_kernel(GatherTable tab, Shape s, const int32_t* __restrict__ counts,
                    int* __restrict__ err)
 {
+    after_previous();
     const int pair = blockIdx.y;
     const int total = tab.kept[pair];  // rows of the pair
     const int cpr = s.d / 8;
@@ -177,8 +179,8 @@ cudaError_t launch_adaptive_select(const Shape& s, int keep_window, const AdaptA
     cudaError_t e = cudaFuncSetAttribute(adaptive_select_kernel,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
-    adaptive_select_kernel<<<s.units / s.hkv, kThreads, sm, st>>>(s, keep_window, a);
-    return cudaGetLastError();
+    return launch_after(adaptive_select_kernel, s.units / s.hkv, kThreads, sm, st, s, keep_window,
+                        a);
 }
 
 cudaError_t launch_gather_flat(const GatherTable& tab, const Shape& s, const int32_t* counts,
@@ -189,8 +191,7 @@ cudaError_t launch_gather_flat(const GatherTable& tab, const Shape& s, const int
     for (int p = 0; p < pairs; ++p) rows = tab.kept[p] > rows ? tab.kept[p] : rows;
     if (rows <= 0) return cudaSuccess;
     dim3 grid((rows * (s.d / 8) + 255) / 256, pairs);
-    gather_flat_kernel<<<grid, 256, 0, st>>>(tab, s, counts, err);
-    return cudaGetLastError();
+    return launch_after(gather_flat_kernel, grid, 256, 0, st, tab, s, counts, err);
 }
 
 }  // namespace bacon

@@ -549,6 +549,7 @@ template <int T, int PER, bool ADAPT>
 __global__ void __launch_bounds__(T, 1024 / T)
 calibrate_select_kernel(Shape s, Calib c, CalibArgs a)
 {
+    after_previous();
     const int u = blockIdx.x;
     calibrate_unit<T, PER, ADAPT>(s, c, a, u, a.lambda + u, a.idx[u / s.hkv]);
 }
@@ -569,6 +570,7 @@ sweep_shared_kernel(Shape s, Calib c, SweepArgs sw, CalibArgs a)
     __shared__ SelectScratch<T> sel_sm;
     __shared__ int ties[32];
     __shared__ float red[2 * 32];
+    after_previous();
     const int u = blockIdx.x, ri = blockIdx.y;
     const int N = s.N, win = c.keep_window ? s.W : 0, n_cand = N - win;
     const int i0 = (int)threadIdx.x * PER;
@@ -608,6 +610,7 @@ calibrate_sweep_kernel(Shape s, CalibTable t, SweepArgs sw, CalibArgs a)
     __shared__ SelectScratch<T> sel_sm;
     __shared__ int ties[32], offsets[32];
     __shared__ float red_s[32], red_v[32];
+    after_previous();
     const int u = blockIdx.x, j = blockIdx.y;
     const Calib& c = t.c[j];
     const int N = s.N, win = c.keep_window ? s.W : 0, n_cand = N - win;
@@ -670,19 +673,18 @@ cudaError_t launch_select_t(const Shape& s, const Calib& c, const CalibArgs& a, 
     cudaError_t e = cudaFuncSetAttribute(calibrate_select_kernel<T, PER, ADAPT>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
-    calibrate_select_kernel<T, PER, ADAPT><<<s.units, T, sm, st>>>(s, c, a);
-    return cudaGetLastError();
+    return launch_after(calibrate_select_kernel<T, PER, ADAPT>, s.units, T, sm, st, s, c, a);
 }
 
 template <int T, int PER>
 cudaError_t launch_sweep_t(const Shape& s, const CalibTable& t, int variants, const SweepArgs& sw,
                            const CalibArgs& a, cudaStream_t st)
 {
-    sweep_shared_kernel<T, PER><<<dim3(s.units, sw.rhos), T, 0, st>>>(s, t.c[0], sw, a);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = launch_after(sweep_shared_kernel<T, PER>, dim3(s.units, sw.rhos), T, 0, st, s,
+                                 t.c[0], sw, a);
     if (e != cudaSuccess) return e;
-    calibrate_sweep_kernel<T, PER><<<dim3(s.units, variants), T, 0, st>>>(s, t, sw, a);
-    return cudaGetLastError();
+    return launch_after(calibrate_sweep_kernel<T, PER>, dim3(s.units, variants), T, 0, st, s, t, sw,
+                        a);
 }
 
 // The launch for a prompt of N tokens: F(T, PER) with the size class above.

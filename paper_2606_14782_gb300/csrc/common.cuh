@@ -74,6 +74,37 @@ __device__ __forceinline__ float key_float(uint32_t k)
 
 // ----------------------------------------------------------- launchers
 
+// Every kernel of the library is launched with programmatic stream
+// serialisation: its blocks may be placed while the previous kernel of the
+// stream finishes, and wait in after_previous() before they touch global
+// memory.  (griddepcontrol.wait returns once that kernel has completed and its
+// writes are visible.  Every block of every kernel waits, so completion is
+// transitive along the stream, and a kernel releases its successor's blocks
+// only after its own wait.)  28 layers of 6528 tokens one by one, five
+// launches each: 1.45 -> 1.13 ms; 28 layers x 4096 tokens at once, five
+// launches: 101 -> 93 us.
+__device__ __forceinline__ void after_previous()
+{
+    asm volatile("griddepcontrol.wait;\n griddepcontrol.launch_dependents;\n" ::: "memory");
+}
+
+template <typename... P, typename... A>
+cudaError_t launch_after(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                         const A&... args)
+{
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 // Calibration + selection per unit (Eqs. 5-17).  The residual of layer j of
 // request rq, kv-head h is read from
 //     Ering + rq * ring_req_stride + (j % ring) * hkv * N + h * N,

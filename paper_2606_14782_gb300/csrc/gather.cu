@@ -11,6 +11,7 @@ namespace {
 __global__ void __launch_bounds__(256)
 gather_kernel(GatherTable tab, Shape s, int* __restrict__ err)
 {
+    after_previous();
     const int u = blockIdx.y;
     const int pair = u / s.hkv, h = u - pair * s.hkv;
     const int kept = tab.kept[pair];
@@ -44,8 +45,7 @@ cudaError_t launch_gather(const GatherTable& tab, const Shape& s, int* err, cuda
     if (kept <= 0) return cudaSuccess;
     const int pieces = kept * (s.d / 8);
     dim3 grid((pieces + 255) / 256, s.units);
-    gather_kernel<<<grid, 256, 0, st>>>(tab, s, err);
-    return cudaGetLastError();
+    return launch_after(gather_kernel, grid, 256, 0, st, tab, s, err);
 }
 
 }  // namespace bacon

@@ -65,6 +65,7 @@ int take_fault()
 __global__ void __launch_bounds__(1024)
 poison_on_error_kernel(int* err, float* B, float* Q, float* E, size_t n)
 {
+    after_previous();
     if (*reinterpret_cast<const volatile int*>(err) == 0) return;
     const float nan = __int_as_float(0x7fc00000);
     for (size_t i = threadIdx.x; i < n; i += blockDim.x) {
@@ -146,11 +147,9 @@ bacon_status bacon_window_scores_noalloc(int kv_heads, int q_heads, int head_dim
     a1.fault = take_fault();
     cudaError_t e = launch_window_stats_tc(a1, m, st);
     if (e == cudaSuccess) e = launch_window_scores_tc(a, m, st);
-    if (e == cudaSuccess) {
-        poison_on_error_kernel<<<1, 1024, 0, st>>>(err, B_out, Q_out, E_out,
-                                                   (size_t)kv_heads * seq_len);
-        e = cudaGetLastError();
-    }
+    if (e == cudaSuccess)
+        e = launch_after(poison_on_error_kernel, 1, 1024, 0, st, err, B_out, Q_out, E_out,
+                         (size_t)kv_heads * seq_len);
     // without that kernel, what this call latched must not reach the next one
     if (e != cudaSuccess) cudaMemsetAsync(err, 0, sizeof(int), st);
     return e == cudaSuccess ? BACON_OK : BACON_ECUDA;

@@ -394,6 +394,14 @@ __global__ void __launch_bounds__(kThreads, 1) window_onepass_kernel(TcArgs a, c
         tc::st_shared_volatile(b.abort(), 0u);
         tc::fence_barrier_init();
     }
+    // the producer starts its loads while the other warps set up (they meet
+    // it at barrier 1, where it only arrives)
+    if (warp == 0) {
+        __syncwarp();
+        tc::named_barrier_arrive(1, kThreads);
+        after_previous();
+        produce<D>(a, maps, L, sm, b);
+    }
     if (threadIdx.x == 32) {
         if (!a.kmaps) tc::tma_prefetch_desc(&maps.k);
         if (!a.qmaps) tc::tma_prefetch_desc(&maps.q);
@@ -403,15 +411,16 @@ __global__ void __launch_bounds__(kThreads, 1) window_onepass_kernel(TcArgs a, c
         tc::tmem_alloc(b.tmem_slot(), 512);
         tc::tmem_relinquish();
     }
-    tc::fence_before_sync();
-    __syncthreads();
-    tc::fence_after_sync();
+    if (warp != 0) {
+        after_previous();
+        tc::fence_before_sync();
+        tc::named_barrier_sync(1, kThreads);
+        tc::fence_after_sync();
+    }
 
-    if (warp == 0)
-        produce<D>(a, maps, L, sm, b);
-    else if (warp == 1) {
+    if (warp == 1) {
         if (tc::elect_one()) issue<D>(a, L, sm, b);
-    } else {
+    } else if (warp >= 2) {
         epilogue<D, SPEC>(a, L, sm, b);
     }
 
@@ -443,8 +452,7 @@ cudaError_t launch_d(const TcArgs& a, const TcMaps& m, cudaStream_t st)
     if (e != cudaSuccess) return e;
     const int sms = num_sms_onepass();
     const int grid = a.s.units < sms ? a.s.units : sms;
-    window_onepass_kernel<D, SPEC><<<grid, kThreads, bytes, st>>>(a, m);
-    return cudaGetLastError();
+    return launch_after(window_onepass_kernel<D, SPEC>, grid, kThreads, bytes, st, a, m);
 }
 
 }  // namespace

@@ -1102,6 +1102,7 @@ __device__ __forceinline__ void epilogue_scores(const TcArgs& a, const Plan& pl,
 __global__ void window_combine_kernel(Shape s, int chunks, const float2* __restrict__ partial,
                                       float* __restrict__ lse2)
 {
+    after_previous();
     const int u = blockIdx.x;
     for (int r = threadIdx.x; r < s.rows; r += blockDim.x)
         lse2[(size_t)u * s.rows + r] =
@@ -1113,6 +1114,7 @@ __global__ void window_combine_kernel(Shape s, int chunks, const float2* __restr
 // [Hq][W] = [Hkv][G W] -> lse2 = LSE log2(e) + log2(G W).
 __global__ void lse_from_prefill_kernel(Shape s, LseTable t, float* __restrict__ lse2)
 {
+    after_previous();
     const int u = blockIdx.x;
     const int pair = u / s.hkv, h = u - pair * s.hkv;
     const float log2_gw = log2f((float)s.rows);
@@ -1166,6 +1168,7 @@ __global__ void __launch_bounds__(kThreads, 1) window_tc_kernel(TcArgs a, Plan p
     if (warp == 0) {
         __syncwarp();
         tc::named_barrier_arrive(1, kThreads);
+        after_previous();
         produce<D, PASS>(a, maps, pl, L, sm, b, jt);
     }
     if (threadIdx.x == 32) {
@@ -1177,6 +1180,7 @@ __global__ void __launch_bounds__(kThreads, 1) window_tc_kernel(TcArgs a, Plan p
         tc::tmem_alloc(b.tmem_slot(), kTmemCols);
         tc::tmem_relinquish();
     }
+    if (warp != 0) after_previous();
     if (PASS == 2 && warp >= 2) {
         // constant operand: 1 in columns 0-2 of every token row (one atom of
         // 8 rows when ones_atom); the bias operand starts zeroed, then takes
@@ -1339,8 +1343,7 @@ cudaError_t launch_impl(const TcArgs& args, const TcMaps& m, cudaStream_t st)
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
     if (e != cudaSuccess) return e;
     const int grid = a.items < sms ? a.items : sms;
-    window_tc_kernel<D, PASS><<<grid, kThreads, bytes, st>>>(a, pl, m);
-    return cudaGetLastError();
+    return launch_after(window_tc_kernel<D, PASS>, grid, kThreads, bytes, st, a, pl, m);
 }
 
 }  // namespace
@@ -1350,16 +1353,14 @@ int window_tc_max_rows() { return 512; }
 cudaError_t launch_lse_from_prefill(const Shape& s, const LseTable& t, float* lse2, cudaStream_t st)
 {
     const int threads = s.rows < 512 ? ((s.rows + 31) / 32) * 32 : 512;
-    lse_from_prefill_kernel<<<s.units, threads, 0, st>>>(s, t, lse2);
-    return cudaGetLastError();
+    return launch_after(lse_from_prefill_kernel, s.units, threads, 0, st, s, t, lse2);
 }
 
 cudaError_t launch_window_combine(const Shape& s, int chunks, const float2* partial,
                                   float* lse2, cudaStream_t st)
 {
     const int threads = s.rows < 512 ? ((s.rows + 31) / 32) * 32 : 512;
-    window_combine_kernel<<<s.units, threads, 0, st>>>(s, chunks, partial, lse2);
-    return cudaGetLastError();
+    return launch_after(window_combine_kernel, s.units, threads, 0, st, s, chunks, partial, lse2);
 }
 
 
