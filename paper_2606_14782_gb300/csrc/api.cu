@@ -46,6 +46,7 @@ bacon_status cuda_fail(cudaError_t e, const char* what)
 bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
 constexpr int kChunkTokens = 1024;  // pass-1 token chunk (multiple of the 128-token tile)
+constexpr size_t kLastBytes = 16ull << 20;  // host path: keys of the last pipelined part, at most
 constexpr int kMaxSeq = 24576;      // calibration keeps 2 x N fp32 in shared memory
 static_assert(kMaxVariants == BACON_MAX_VARIANTS, "variant table size");
 
@@ -95,6 +96,7 @@ struct bacon_ctx {
     uint2* key_range = nullptr;
     float2* moments = nullptr;  // sweep: B~'s moment sums per distinct rho
     int* err = nullptr;
+    int* h_err = nullptr;  // page-locked copy of the error word (host path)
     int last_units = 0, last_N = 0;
     // staging buffers of bacon_compress_host
     void* hq_buf = nullptr;
@@ -285,6 +287,8 @@ void free_ctx_buffers(bacon_ctx* c)
     c->h2d = c->d2h = nullptr;
     if (c->maps_ev) cudaEventDestroy(c->maps_ev);
     if (c->h_maps) cudaFreeHost(c->h_maps);
+    if (c->h_err) cudaFreeHost(c->h_err);
+    c->h_err = nullptr;
     if (c->d_maps) cudaFree(c->d_maps);
     c->maps_ev = nullptr;
     c->h_maps = nullptr;
@@ -412,8 +416,11 @@ bacon_status window_passes(bacon_ctx* c, const Shape& s, const void* const* q,
     return BACON_OK;
 }
 
-// The whole step.  layer_budget[l] is the budget of layer l (window
-// included); idx[pair] receives the pair's [Hkv][min(budget, N)] positions.
+// The whole step of layers [layer0, layer0 + nlayers) of R requests (R = 1
+// unless that is every layer), whose units start at unit0 of the scratch and
+// whose persistence reads the residuals of the layers before from there.
+// layer_budget[l] is the budget of layer layer0 + l (window included);
+// idx[pair] receives the pair's [Hkv][min(budget, N)] positions.
 // With adaptive = true (uniform budget), the heads of each layer share the
 // budget (AdaKV-style, g = guaranteed candidates per head first): idx[pair]
 // and the K/V outputs are flat per pair, heads in order, with per-head kept
@@ -423,19 +430,21 @@ bacon_status compress_device(bacon_ctx* c, int R, const void* const* q, const vo
                              void* const* ko, void* const* vo, int32_t* const* idx,
                              cudaStream_t st, bool adaptive = false, int guaranteed = 0,
                              int32_t* counts = nullptr, size_t unit0 = 0,
-                             const float* const* prefill_lse = nullptr, int map0 = 0)
+                             const float* const* prefill_lse = nullptr, int layer0 = 0,
+                             int nlayers = 0)
 {
-    const int pairs = R * c->layers;
-    const Shape s = shape_of(c, c->layers, R, N);
+    if (nlayers == 0) nlayers = c->layers;
+    const int pairs = R * nlayers, map0 = (int)(unit0 / c->hkv);
+    const Shape s = shape_of(c, nlayers, R, N);
     float* B = c->B + unit0 * N;
-    float* E = c->E + unit0 * N;
+    float* E = c->E + (unit0 - (size_t)layer0 * c->hkv) * N;  // layer 0's
     float* S = c->S + unit0 * N;
     float* lam = c->lam + unit0;
 
     GatherTable gt;
     CalibArgs a;
     for (int i = 0; i < pairs; ++i) {
-        const int budget = layer_budget[i % c->layers];
+        const int budget = layer_budget[i % nlayers];
         gt.k[i] = static_cast<const uint16_t*>(k[i]);
         gt.v[i] = static_cast<const uint16_t*>(v[i]);
         gt.ko[i] = static_cast<uint16_t*>(ko[i]);
@@ -454,7 +463,7 @@ bacon_status compress_device(bacon_ctx* c, int R, const void* const* q, const vo
     a.Ering = E;
     a.ring = c->layers;
     a.ring_req_stride = (long long)c->layers * c->hkv * N;
-    a.layer0 = 0;
+    a.layer0 = layer0;
     a.S = S;
     a.V = c->p.keep_scores ? c->V + unit0 * N : nullptr;
     a.Bp = c->p.keep_scores ? c->Bp + unit0 * N : nullptr;
@@ -694,6 +703,8 @@ bacon_status bacon_init(bacon_ctx** out, int layers, int kv_heads, int q_heads, 
     if (e == cudaSuccess)
         e = cudaHostAlloc(reinterpret_cast<void**>(&c->h_maps), 2 * kMaxPairs * sizeof(CUtensorMap),
                           cudaHostAllocDefault);
+    if (e == cudaSuccess)
+        e = cudaHostAlloc(reinterpret_cast<void**>(&c->h_err), sizeof(int), cudaHostAllocDefault);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->maps_ev, cudaEventDisableTiming);
     if (e != cudaSuccess) {
         cudaGetLastError();
@@ -1077,11 +1088,37 @@ bacon_status bacon_compress_host(bacon_ctx* ctx, int requests, const void* q_win
         ctx->ev_in.push_back(a);
         ctx->ev_done.push_back(b);
     }
-    // Requests are pipelined: every upload is queued on one copy stream, a
-    // request is compressed on the caller's stream as soon as its inputs have
-    // landed, and its outputs go back on a second copy stream while the next
-    // request computes.
+    // Parts are pipelined: every upload is queued on one copy stream, a part
+    // is compressed on the caller's stream as soon as its inputs have landed
+    // (layers in order: persistence reads the residuals of the layers
+    // before), and its outputs go back on a second copy stream while the next
+    // part computes.  A part is a whole request, except that the last request
+    // is halved again and again: only what follows the last upload is not
+    // hidden behind the link, one small part's compression and download.
+    // (Every further part costs about 12 us of copy and kernel overheads, so
+    // the halving ends at kLastBytes of keys.)  28 layers x 4096 tokens, one
+    // request: 968 us whole, 826 halved; equal parts of 32, 16 and 8 MB of
+    // keys took 851, 895 and 1038 us.
     const int L = ctx->layers;
+    struct Part {
+        int r, l0, n;
+    };
+    Part parts[kMaxPairs + 32];  // requests, and at most 9 halvings of at most 256 layers
+    size_t nparts = 0;
+    for (int r = 0; r + 1 < requests; ++r) parts[nparts++] = {r, 0, L};
+    for (int l0 = 0; l0 < L;) {
+        const int left = L - l0;
+        const int n = kv_pair * 2 * left <= kLastBytes ? left : (left + 1) / 2;
+        parts[nparts++] = {requests - 1, l0, n};
+        l0 += n;
+    }
+    while (ctx->ev_in.size() < nparts) {
+        cudaEvent_t a = nullptr, b = nullptr;
+        BACON_CUDA(cudaEventCreateWithFlags(&a, cudaEventDisableTiming), "event");
+        BACON_CUDA(cudaEventCreateWithFlags(&b, cudaEventDisableTiming), "event");
+        ctx->ev_in.push_back(a);
+        ctx->ev_done.push_back(b);
+    }
     const char* qh = static_cast<const char*>(q_win);
     const char* kh = static_cast<const char*>(k);
     const char* vh = static_cast<const char*>(v);
@@ -1103,44 +1140,54 @@ bacon_status bacon_compress_host(bacon_ctx* ctx, int requests, const void* q_win
     // engine.)
     BACON_CUDA(cudaEventRecord(ctx->ev_done[0], cs), "event");  // uploads start after earlier work
     BACON_CUDA(cudaStreamWaitEvent(ctx->h2d, ctx->ev_done[0], 0), "event wait");
-    for (int r = 0; r < requests; ++r) {
-        const size_t qb = q_pair * L * 2, kb = kv_pair * L * 2;
-        BACON_CUDA(cudaMemcpyAsync(static_cast<char*>(ctx->hq_buf) + r * qb, qh + r * qb, qb,
-                                   cudaMemcpyHostToDevice, ctx->h2d), "query upload");
-        BACON_CUDA(cudaMemcpyAsync(static_cast<char*>(ctx->hk_buf) + r * kb, kh + r * kb, kb,
+    for (size_t e = 0; e < nparts; ++e) {
+        const int r = parts[e].r, l0 = parts[e].l0, n = parts[e].n;
+        const size_t pair0 = (size_t)r * L + l0;
+        const size_t q0 = q_pair * pair0 * 2, k0 = kv_pair * pair0 * 2;
+        const size_t qb = q_pair * L * 2, kb = kv_pair * n * 2;
+        if (l0 == 0)  // the request's queries, in one copy
+            BACON_CUDA(cudaMemcpyAsync(static_cast<char*>(ctx->hq_buf) + q0, qh + q0, qb,
+                                       cudaMemcpyHostToDevice, ctx->h2d), "query upload");
+        BACON_CUDA(cudaMemcpyAsync(static_cast<char*>(ctx->hk_buf) + k0, kh + k0, kb,
                                    cudaMemcpyHostToDevice, ctx->h2d), "key upload");
         if (!v_dev)
-            BACON_CUDA(cudaMemcpyAsync(static_cast<char*>(ctx->hv_buf) + r * kb, vh + r * kb, kb,
+            BACON_CUDA(cudaMemcpyAsync(static_cast<char*>(ctx->hv_buf) + k0, vh + k0, kb,
                                        cudaMemcpyHostToDevice, ctx->h2d), "value upload");
-        BACON_CUDA(cudaEventRecord(ctx->ev_in[r], ctx->h2d), "event");
+        BACON_CUDA(cudaEventRecord(ctx->ev_in[e], ctx->h2d), "event");
     }
 
     std::vector<int> budgets(L, budget);
     int32_t* idx_pairs[kMaxPairs];
     for (int i = 0; i < pairs; ++i) idx_pairs[i] = ctx->hidx_buf + (size_t)i * ctx->hkv * kept;
-    for (int r = 0; r < requests; ++r) {
-        BACON_CUDA(cudaStreamWaitEvent(cs, ctx->ev_in[r], 0), "event wait");
-        rc = compress_device(ctx, 1, qs + r * L, ks + r * L, vs + r * L, seq_len, budgets.data(),
-                             kos + r * L, vos + r * L, idx_pairs + r * L, cs, false, 0, nullptr,
-                             (size_t)r * L * ctx->hkv, nullptr, r * L);
+    for (size_t e = 0; e < nparts; ++e) {
+        const int l0 = parts[e].l0, n = parts[e].n;
+        const size_t pair0 = (size_t)parts[e].r * L + l0;
+        BACON_CUDA(cudaStreamWaitEvent(cs, ctx->ev_in[e], 0), "event wait");
+        rc = compress_device(ctx, 1, qs + pair0, ks + pair0, vs + pair0, seq_len, budgets.data(),
+                             kos + pair0, vos + pair0, idx_pairs + pair0, cs, false, 0, nullptr,
+                             pair0 * ctx->hkv, nullptr, l0, n);
         if (rc != BACON_OK) return rc;
-        BACON_CUDA(cudaEventRecord(ctx->ev_done[r], cs), "event");
-        BACON_CUDA(cudaStreamWaitEvent(ctx->d2h, ctx->ev_done[r], 0), "event wait");
-        const size_t ob = o_pair * L * 2, ib = (size_t)L * ctx->hkv * kept * 4;
-        BACON_CUDA(cudaMemcpyAsync(static_cast<char*>(k_out) + r * ob,
-                                   static_cast<char*>(ctx->hko_buf) + r * ob, ob,
+        BACON_CUDA(cudaEventRecord(ctx->ev_done[e], cs), "event");
+        BACON_CUDA(cudaStreamWaitEvent(ctx->d2h, ctx->ev_done[e], 0), "event wait");
+        const size_t o0 = o_pair * pair0 * 2, ob = o_pair * n * 2;
+        const size_t i0 = pair0 * ctx->hkv * kept * 4, ib = (size_t)n * ctx->hkv * kept * 4;
+        BACON_CUDA(cudaMemcpyAsync(static_cast<char*>(k_out) + o0,
+                                   static_cast<char*>(ctx->hko_buf) + o0, ob,
                                    cudaMemcpyDeviceToHost, ctx->d2h), "key download");
-        BACON_CUDA(cudaMemcpyAsync(static_cast<char*>(v_out) + r * ob,
-                                   static_cast<char*>(ctx->hvo_buf) + r * ob, ob,
+        BACON_CUDA(cudaMemcpyAsync(static_cast<char*>(v_out) + o0,
+                                   static_cast<char*>(ctx->hvo_buf) + o0, ob,
                                    cudaMemcpyDeviceToHost, ctx->d2h), "value download");
-        BACON_CUDA(cudaMemcpyAsync(reinterpret_cast<char*>(idx_out) + r * ib,
-                                   reinterpret_cast<char*>(ctx->hidx_buf) + r * ib, ib,
+        BACON_CUDA(cudaMemcpyAsync(reinterpret_cast<char*>(idx_out) + i0,
+                                   reinterpret_cast<char*>(ctx->hidx_buf) + i0, ib,
                                    cudaMemcpyDeviceToHost, ctx->d2h), "index download");
     }
     (void)idx_count;
+    // the error word comes with the outputs (the downloads follow every
+    // kernel of the call); only a latched error takes the way of bacon_sync
+    BACON_CUDA(cudaMemcpyAsync(ctx->h_err, ctx->err, sizeof(int), cudaMemcpyDeviceToHost, ctx->d2h),
+               "error flag download");
     BACON_CUDA(cudaStreamSynchronize(ctx->d2h), "host-path synchronisation");
-    BACON_CUDA(cudaStreamSynchronize(cs), "host-path synchronisation");
-    return bacon_sync(ctx, stream);
+    return *ctx->h_err ? bacon_sync(ctx, stream) : BACON_OK;
 }
 
 bacon_status bacon_get_scores(bacon_ctx* ctx, bacon_score_kind kind, float* out, size_t count,

@@ -80,3 +80,26 @@ def test_scores_out_at_any_float_alignment(offset):
     assert (buf[:offset] == 7.0).all() and (buf[offset + hkv * n:] == 7.0).all()
     st.close()
     ctx.close()
+
+
+@pytest.mark.parametrize("layers,requests,seq_len", [(7, 2, 8192), (9, 1, 4099), (1, 1, 16384)])
+def test_host_path_in_parts(layers, requests, seq_len):
+    """Keys beyond one pipelined part: the last request goes in halves, and
+    persistence reads the residuals of the parts before."""
+    hkv, d, w, budget = 3, 128, 16, 200
+    wl = workloads.CONFIGS["tiny"].with_(
+        layers=layers, requests=requests, q_heads=2 * hkv, kv_heads=hkv, head_dim=d,
+        seq_len=seq_len, window=w, visual=(16, seq_len - 200))
+    x = workloads.generate(wl, seed=21, device="cuda")
+    ctx = bacon.Context(layers, hkv, 2 * hkv, d, w, 7, budget, max_seq_len=seq_len,
+                        max_requests=requests, keep_scores=1)
+    want = ctx.compress_all_layers(x.qwin, x.k, x.v, budget)
+    scores = {n: ctx.scores(n).clone() for n in ("B", "E", "V", "S", "lambda")}
+    qh, kh, vh = (t.cpu().pin_memory() for t in (x.qwin, x.k, x.v))
+    for _ in range(2):
+        got = ctx.compress_host(qh, kh, vh, budget)
+        for a, b in zip(got, want):
+            assert torch.equal(a, b.cpu())
+        for n, s in scores.items():
+            assert torch.equal(ctx.scores(n), s), n
+    ctx.close()
