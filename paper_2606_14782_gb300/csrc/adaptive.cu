@@ -86,9 +86,9 @@ adaptive_select_kernel(Shape s, int keep_window, AdaptArgs a)
         }
         sel = select_each<kThreads>(each_key, rest, sel_sm, kmin, kmax);
         if (!sel.all_ties_in()) {
-            int eq = 0, total;
+            int eq = 0;
             each_key([&](bool in, uint32_t key) { eq += in && key == sel.tau; });
-            rank = block_exclusive_scan<kThreads>(eq, ties, total);
+            rank = block_exclusive_scan<kThreads>(eq, ties).x;
         }
     }
     // 3. the members of every run, then their places
@@ -111,8 +111,9 @@ adaptive_select_kernel(Shape s, int keep_window, AdaptArgs a)
         kept_map[r] = (uint8_t)m;
         mine += __popc(m);
     });
-    int total;
-    int pos = block_exclusive_scan<kThreads>(mine, offsets, total);
+    const int2 at = block_exclusive_scan<kThreads>(mine, offsets);
+    int pos = at.x;
+    const int total = at.y;
     int32_t* out = a.idx[pair];
     int32_t* counts = a.counts + (size_t)pair * H;
     for (int r = r0; r < r1; ++r) {

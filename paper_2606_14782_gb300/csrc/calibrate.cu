@@ -74,14 +74,6 @@ __device__ __forceinline__ void block_sums(float (&v)[NV], float* red)
         for (int i = 0; i < NV; ++i) v[i] += __shfl_xor_sync(0xffffffffu, v[i], o);
 }
 
-// Ask L2 to fetch the n floats at p (one prefetch per 128-byte line, every
-// address inside the array), so that later loads of them hit L2.
-__device__ __forceinline__ void prefetch_l2(const float* p, int n)
-{
-    for (int i = (int)threadIdx.x * 32; i < n; i += (int)blockDim.x * 32)
-        asm volatile("prefetch.global.L2 [%0];" ::"l"(p + i));
-}
-
 // dst[i0 + k] = x[k] for the positions below n.
 template <int PER>
 __device__ __forceinline__ void store_run(float* dst, int i0, int n, const float* x)
@@ -127,10 +119,10 @@ __device__ __forceinline__ int ties_before(const float* x, int nv, const SelectR
                                            int* warp_sums)
 {
     if (sel.all_ties_in()) return 0;
-    int eq = 0, total;
+    int eq = 0;
 #pragma unroll
     for (int k = 0; k < PER; ++k) eq += k < nv && float_key(x[k]) == sel.tau;
-    return block_exclusive_scan<T>(eq, warp_sums, total);
+    return block_exclusive_scan<T>(eq, warp_sums).x;
 }
 
 // The residual E of the thread's run into x (0 at and past N), added to v
@@ -242,33 +234,71 @@ __device__ __forceinline__ void residual_and_coherence(const float* __restrict__
     coherence_any<PER>(Ec, i0, N, r, v);
 }
 
-// The evidence V = E + L + T of the thread's run (Eqs. 5-11) into v, 0 at and
-// past N; x is scratch for PER floats.  E_of(j) is layer j's residuals.
-template <int PER, typename EFn>
-__device__ __forceinline__ void evidence_run(const Calib& c, EFn E_of, int layer, int i0, int N,
-                                             float* x, float* v)
+// The residuals that a unit reads: layer l's row is at base + (l % ring) *
+// layer_stride.
+struct Residuals {
+    const float* base;
+    long long layer_stride;
+    int ring;
+    __device__ __forceinline__ const float* row(int l) const
+    {
+        return base + (long long)(l % ring) * layer_stride;
+    }
+};
+
+__device__ __forceinline__ Residuals residuals_of(const CalibArgs& a, const Shape& s, int rq, int h)
 {
-    const float* Ec = E_of(layer);
+    return {a.Ering + (long long)rq * a.ring_req_stride + (long long)h * s.N,
+            (long long)s.hkv * s.N, a.ring};
+}
+
+// v += the runs of layers [l0, l0 + n), in layer order; AHEAD layers' loads
+// are in flight together.
+template <int PER, int AHEAD>
+__device__ __forceinline__ void add_layers(const Residuals& E, int l0, int n, int i0, int N,
+                                           float* v)
+{
+    int slot = l0 % E.ring;
+    if ((N & 3) == 0 && i0 + PER <= N) {
+#pragma unroll AHEAD
+        for (int j = 0; j < n; ++j) {
+            const float4* p = reinterpret_cast<const float4*>(E.base + slot * E.layer_stride + i0);
+#pragma unroll
+            for (int q = 0; q < PER / 4; ++q) {
+                const float4 e = __ldg(p + q);
+                v[4 * q] += e.x;
+                v[4 * q + 1] += e.y;
+                v[4 * q + 2] += e.z;
+                v[4 * q + 3] += e.w;
+            }
+            if (++slot == E.ring) slot = 0;
+        }
+    } else {
+#pragma unroll 1
+        for (int j = 0; j < n; ++j) {
+            const float* p = E.base + slot * E.layer_stride;
+#pragma unroll
+            for (int k = 0; k < PER; ++k)
+                if (i0 + k < N) v[k] += __ldg(p + i0 + k);
+            if (++slot == E.ring) slot = 0;
+        }
+    }
+}
+
+// The evidence V = E + L + T of the thread's run (Eqs. 5-11) into v, 0 at and
+// past N; x is scratch for PER floats.
+template <int PER>
+__device__ __forceinline__ void evidence_run(const Calib& c, const Residuals& E, int layer, int i0,
+                                             int N, float* x, float* v)
+{
+    const float* Ec = E.row(layer);
 #pragma unroll
     for (int k = 0; k < PER; ++k) v[k] = 0.f;
     // persistence: mean of E over the preceding min(m, l) layers (Eqs. 8-9)
     if (c.use_T) {
         const int nprev = min(c.m, layer);
         const float inv_prev = nprev > 0 ? 1.f / (float)nprev : 0.f;
-        // a layer's run in chunks of at most 16 (V and one chunk in registers)
-        constexpr int CH = PER <= 16 ? PER : PER / 2;
-        static_assert(PER % CH == 0 && CH % 4 == 0, "chunks of whole 16-byte loads");
-        constexpr int kAhead = PER <= 8 ? 4 : 1;  // layers whose loads are in flight together
-#pragma unroll kAhead
-        for (int j = layer - nprev; j < layer; ++j) {
-#pragma unroll
-            for (int c0 = 0; c0 < PER; c0 += CH) {
-                float e[CH];
-                load_run<CH>(E_of(j), i0 + c0, N, e);
-#pragma unroll
-                for (int k = 0; k < CH; ++k) v[c0 + k] += e[k];
-            }
-        }
+        add_layers<PER, (PER <= 8 ? 4 : (PER <= 16 ? 2 : 1))>(E, layer - nprev, nprev, i0, N, v);
 #pragma unroll
         for (int k = 0; k < PER; ++k) v[k] *= inv_prev;
     }
@@ -368,25 +398,21 @@ __device__ __forceinline__ float lambda_of(const Calib& c, int M, uint32_t mem, 
     return c.gamma * stdb / (stdv + c.eps);
 }
 
-// Eq. 17: the `keep` best candidates by the scores in b (key range skmin,
-// skmax), ascending, then the window.
+// Eq. 17's output: the members (`mem`, `keep` of them in all), ascending,
+// then the window.
 template <int T, int PER>
-__device__ __forceinline__ void emit_best(const float* b, int i0, int nv, int n_cand, int keep,
-                                          int win, int N, uint32_t skmin, uint32_t skmax,
-                                          SelectScratch<T>& sel_sm, int* ties, int* offsets,
-                                          int32_t* out, int* err)
+__device__ __forceinline__ void emit(uint32_t mem, int i0, int n_cand, int keep, int win, int N,
+                                     int* offsets, int32_t* out, int* err)
 {
     if (keep >= n_cand) {
         for (int i = threadIdx.x; i < n_cand; i += T) out[i] = i;
     } else if (keep > 0) {
-        const SelectResult sel = select_runs<T, PER>(b, nv, keep, sel_sm, skmin, skmax);
-        const uint32_t mem = members<PER>(b, nv, sel, ties_before<T, PER>(b, nv, sel, ties));
-        int total;
-        int pos = block_exclusive_scan<T>(__popc(mem), offsets, total);
+        const int2 at = block_exclusive_scan<T>(__popc(mem), offsets);
+        int pos = at.x;
 #pragma unroll
         for (int k = 0; k < PER; ++k)
             if ((mem >> k) & 1u) out[pos++] = i0 + k;
-        if (threadIdx.x == 0 && total != keep && err) atomicCAS(err, 0, 2);
+        if (threadIdx.x == 0 && at.y != keep && err) atomicCAS(err, 0, 2);
     }
     for (int w = threadIdx.x; w < win; w += T) out[keep + w] = N - win + w;
 }
@@ -403,8 +429,10 @@ __device__ __forceinline__ int match_count(int rho, int budget, int N, int win, 
 // (may be null) receives lambda; idx_pair is the pair's [Hkv][kept] output.
 // N <= T PER.  The thread's run of the pooled backbone (then of the final
 // score: the keys of the two selections) stays in registers, and so does V
-// where a run is 8 positions; longer runs form V after the first selection,
-// with the backbone parked in the thread's own column of shared memory.
+// where a run is 8 positions; longer runs park V in the thread's own column
+// of shared memory while the first selection needs the registers.  The two
+// selections are two turns of one loop, so that the second finds its code in
+// the instruction cache.
 // ADAPT: the head's guaranteed share and its key range for the adaptive
 // selection take the place of Eq. 17.
 template <int T, int PER, bool ADAPT>
@@ -429,120 +457,114 @@ __device__ __forceinline__ void calibrate_unit(const Shape& s, const Calib& c, c
     const int nv = max(0, min(PER, n_cand - i0));  // this thread's candidates
 
     float b[PER];  // pooled backbone B~, then the final score S
-    uint32_t skmin = 0xffffffffu, skmax = 0u;  // key range of S over the candidates
-    auto E_of = [&](int j) -> const float* {
-        return a.Ering + (long long)rq * a.ring_req_stride +
-               (long long)(j % a.ring) * s.hkv * N + (long long)h * N;
-    };
-
+    float v[PER];  // evidence V
+    uint32_t kmin = 0xffffffffu, kmax = 0u;  // range of b's keys over the candidates
+    int M = 0;
     if (a.compute_scores) {
-        const float* Bu = a.B + (size_t)u * N;
-        float x[PER], v[PER];
-        load_run<PER>(Bu, i0, N, b);
-        if (kPark) {
-            // the residuals are read only after the first selection: start
-            // bringing them into L2 now
-            prefetch_l2(E_of(layer), N);
-            if (c.use_T)
-                for (int j = layer - min(c.m, layer); j < layer; ++j) prefetch_l2(E_of(j), N);
-        } else {
-            evidence_run<PER>(c, E_of, layer, i0, N, x, v);
-        }
-        uint32_t kmin = 0xffffffffu, kmax = 0u;  // key range of B~ over the candidates
-        pool_run<PER>(Bu, i0, n_cand, c.pool / 2, b, kmin, kmax);
-        if (a.Bp) store_run<PER>(a.Bp + (size_t)u * N, i0, N, b);
-
-        // ---- the M best candidates by B~ (Eq. 12)
-        const int M = match_count(c.rho, a.calib_budget[pair], N, win, n_cand);
-        uint32_t mem = 0u;
-        float pb = 0.f;
-        if (M > 0) {
-            const SelectResult sel = select_runs<T, PER>(b, nv, M, sel_sm, kmin, kmax);
-            mem = members<PER>(b, nv, sel, ties_before<T, PER>(b, nv, sel, ties[0]));
-            pb = key_float(sel.tau);
-        }
-        if (kPark) {
-#pragma unroll
-            for (int k = 0; k < PER; ++k) sm[k * T + threadIdx.x] = b[k];
-            evidence_run<PER>(c, E_of, layer, i0, N, x, v);
-#pragma unroll
-            for (int k = 0; k < PER; ++k) b[k] = sm[k * T + threadIdx.x];
+        {
+            float x[PER];
+            evidence_run<PER>(c, residuals_of(a, s, rq, h), layer, i0, N, x, v);
         }
         if (a.V) store_run<PER>(a.V + (size_t)u * N, i0, N, v);
-
-        // ---- lambda over the M members (Eqs. 13-15)
-        float lam = 0.f;
-        if (M > 0) {
-            float acc[3] = {0.f, 0.f, 0.f};
+        if (kPark) {
 #pragma unroll
-            for (int k = 0; k < PER; ++k) {
-                if ((mem >> k) & 1u) {
-                    const float db = b[k] - pb;
-                    acc[0] += db;
-                    acc[1] = fmaf(db, db, acc[1]);
-                    acc[2] += v[k];
-                }
-            }
-            block_sums<T, 3>(acc, red_b);
-            lam = lambda_of<T, PER>(c, M, mem, acc[0], acc[1], acc[2], v, red_v);
+            for (int k = 0; k < PER; ++k) sm[k * T + threadIdx.x] = v[k];
         }
-        if (threadIdx.x == 0 && lam_out) *lam_out = lam;
-        // ---- Eq. 16 over the candidates (0 elsewhere)
-#pragma unroll
-        for (int k = 0; k < PER; ++k) {
-            if (k < nv) {
-                b[k] = fmaf(lam, v[k], b[k]);
-                skmin = min(skmin, float_key(b[k]));
-                skmax = max(skmax, float_key(b[k]));
-            }
-        }
-        if (a.write_S) store_run<PER>(a.S + (size_t)u * N, i0, N, b);
-        if (a.S_copy) store_run<PER>(a.S_copy + (size_t)u * N, i0, N, b);
+        const float* Bu = a.B + (size_t)u * N;
+        load_run<PER>(Bu, i0, N, b);
+        pool_run<PER>(Bu, i0, n_cand, c.pool / 2, b, kmin, kmax);
+        if (a.Bp) store_run<PER>(a.Bp + (size_t)u * N, i0, N, b);
+        M = match_count(c.rho, a.calib_budget[pair], N, win, n_cand);
     } else {
         load_run<PER>(a.S + (size_t)u * N, i0, N, b);
 #pragma unroll
         for (int k = 0; k < PER; ++k) {
             if (k < nv) {
-                skmin = min(skmin, float_key(b[k]));
-                skmax = max(skmax, float_key(b[k]));
+                kmin = min(kmin, float_key(b[k]));
+                kmax = max(kmax, float_key(b[k]));
             }
         }
     }
 
-    if constexpr (ADAPT) {
-        // adaptive head budgets: the head's own best candidates as a bitmap of
-        // positions, and the key range of its scores
-        const int sure = min(a.guaranteed, keep);
+    // turn 0: the M best candidates by B~ (Eq. 12), lambda, S; turn 1: the
+    // best by S
+#pragma unroll 1
+    for (int turn = a.compute_scores ? 0 : 1; turn < 2; ++turn) {
+        int k_best = M;
+        if (turn == 1) {
+            if (!ADAPT && !a.do_select) return;
+            k_best = ADAPT ? min(a.guaranteed, keep) : keep;
+            if (keep >= n_cand) k_best = 0;  // every candidate is kept
+        }
         uint32_t mem = 0u;
-        if (keep >= n_cand) {
-            mem = (1u << nv) - 1u;
-        } else if (sure > 0) {
-            const SelectResult sel = select_runs<T, PER>(b, nv, sure, sel_sm, skmin, skmax);
-            mem = members<PER>(b, nv, sel, ties_before<T, PER>(b, nv, sel, ties[1]));
+        float pb = 0.f;
+        if (k_best > 0) {
+            const SelectResult sel = select_runs<T, PER>(b, nv, k_best, sel_sm, kmin, kmax);
+            mem = members<PER>(b, nv, sel, ties_before<T, PER>(b, nv, sel, ties[turn]));
+            pb = key_float(sel.tau);
         }
-        uint8_t* map = a.taken + (size_t)u * a.taken_stride;
+        if (turn == 0) {
+            if (kPark) {
 #pragma unroll
-        for (int q = 0; q < PER / 8; ++q)
-            if (i0 + 8 * q < n_cand) map[i0 / 8 + q] = (uint8_t)(mem >> (8 * q));
-        __shared__ uint32_t ranges[2][32];
-        const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-        skmin = __reduce_min_sync(0xffffffffu, skmin);
-        skmax = __reduce_max_sync(0xffffffffu, skmax);
-        if (lane == 0) {
-            ranges[0][warp] = skmin;
-            ranges[1][warp] = skmax;
+                for (int k = 0; k < PER; ++k) v[k] = sm[k * T + threadIdx.x];
+            }
+            // lambda over the M members (Eqs. 13-15)
+            float lam = 0.f;
+            if (M > 0) {
+                float acc[3] = {0.f, 0.f, 0.f};
+#pragma unroll
+                for (int k = 0; k < PER; ++k) {
+                    if ((mem >> k) & 1u) {
+                        const float db = b[k] - pb;
+                        acc[0] += db;
+                        acc[1] = fmaf(db, db, acc[1]);
+                        acc[2] += v[k];
+                    }
+                }
+                block_sums<T, 3>(acc, red_b);
+                lam = lambda_of<T, PER>(c, M, mem, acc[0], acc[1], acc[2], v, red_v);
+            }
+            if (threadIdx.x == 0 && lam_out) *lam_out = lam;
+            // Eq. 16 over the candidates (0 elsewhere)
+            kmin = 0xffffffffu;
+            kmax = 0u;
+#pragma unroll
+            for (int k = 0; k < PER; ++k) {
+                if (k < nv) {
+                    b[k] = fmaf(lam, v[k], b[k]);
+                    kmin = min(kmin, float_key(b[k]));
+                    kmax = max(kmax, float_key(b[k]));
+                }
+            }
+            if (a.write_S) store_run<PER>(a.S + (size_t)u * N, i0, N, b);
+            if (a.S_copy) store_run<PER>(a.S_copy + (size_t)u * N, i0, N, b);
+        } else if constexpr (ADAPT) {
+            // the head's own best candidates as a bitmap of positions, and the
+            // key range of its scores
+            if (keep >= n_cand) mem = (1u << nv) - 1u;
+            uint8_t* map = a.taken + (size_t)u * a.taken_stride;
+#pragma unroll
+            for (int q = 0; q < PER / 8; ++q)
+                if (i0 + 8 * q < n_cand) map[i0 / 8 + q] = (uint8_t)(mem >> (8 * q));
+            __shared__ uint32_t ranges[2][32];
+            const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+            kmin = __reduce_min_sync(0xffffffffu, kmin);
+            kmax = __reduce_max_sync(0xffffffffu, kmax);
+            if (lane == 0) {
+                ranges[0][warp] = kmin;
+                ranges[1][warp] = kmax;
+            }
+            __syncthreads();
+            if (warp == 0) {
+                kmin = __reduce_min_sync(0xffffffffu, lane < T / 32 ? ranges[0][lane] : 0xffffffffu);
+                kmax = __reduce_max_sync(0xffffffffu, lane < T / 32 ? ranges[1][lane] : 0u);
+                if (lane == 0) a.key_range[u] = make_uint2(kmin, kmax);
+            }
+        } else {
+            emit<T, PER>(mem, i0, n_cand, keep, win, N, offsets, idx_pair + (size_t)h * kept_total,
+                         a.err);
         }
-        __syncthreads();
-        if (warp == 0) {
-            skmin = __reduce_min_sync(0xffffffffu, lane < T / 32 ? ranges[0][lane] : 0xffffffffu);
-            skmax = __reduce_max_sync(0xffffffffu, lane < T / 32 ? ranges[1][lane] : 0u);
-            if (lane == 0) a.key_range[u] = make_uint2(skmin, skmax);
-        }
-        return;
     }
-    if (a.do_select)
-        emit_best<T, PER>(b, i0, nv, n_cand, keep, win, N, skmin, skmax, sel_sm, ties[1], offsets,
-                          idx_pair + (size_t)h * kept_total, a.err);
 }
 
 template <int T, int PER, bool ADAPT>
@@ -630,10 +652,7 @@ calibrate_sweep_kernel(Shape s, CalibTable t, SweepArgs sw, CalibArgs a)
             if (i0 + 8 * q < n_cand) mem |= (uint32_t)map[i0 / 8 + q] << (8 * q);
     }
     float x[PER], v[PER], b[PER];
-    evidence_run<PER>(c, [&](int l) -> const float* {
-        return a.Ering + (long long)rq * a.ring_req_stride +
-               (long long)(l % a.ring) * s.hkv * N + (long long)h * N;
-    }, layer, i0, N, x, v);
+    evidence_run<PER>(c, residuals_of(a, s, rq, h), layer, i0, N, x, v);
     load_run<PER>(sw.pooled + (size_t)u * N, i0, N, b);
     float lam = 0.f;
     if (M > 0) {
@@ -655,9 +674,14 @@ calibrate_sweep_kernel(Shape s, CalibTable t, SweepArgs sw, CalibArgs a)
             skmax = max(skmax, float_key(b[k]));
         }
     }
-    emit_best<T, PER>(b, i0, nv, n_cand, kept_total - win, win, N, skmin, skmax, sel_sm, ties,
-                      offsets, a.idx[pair] + (size_t)j * a.idx_variant_stride + (size_t)h * kept_total,
-                      a.err);
+    const int keep = kept_total - win;
+    mem = 0u;
+    if (keep > 0 && keep < n_cand) {
+        const SelectResult sel = select_runs<T, PER>(b, nv, keep, sel_sm, skmin, skmax);
+        mem = members<PER>(b, nv, sel, ties_before<T, PER>(b, nv, sel, ties));
+    }
+    emit<T, PER>(mem, i0, n_cand, keep, win, N, offsets,
+                 a.idx[pair] + (size_t)j * a.idx_variant_stride + (size_t)h * kept_total, a.err);
 }
 
 template <int T, int PER>

@@ -22,11 +22,14 @@ struct SelectResult {
     __device__ __forceinline__ bool all_ties_in() const { return need == count_eq; }
 };
 
-// Exclusive prefix sum of one int per thread, in thread order; total receives
-// the sum.  One block barrier: every warp scans the warps' sums itself.
-// warp_sums holds 32 ints and is not used again before the next barrier.
+// Exclusive prefix sum of one int per thread, in thread order (x), and the
+// sum of all (y).  One block barrier: every warp scans the warps' sums itself.
+// warp_sums holds 32 ints and is not used again before the next barrier.  A
+// call and not inlined: the kernels here run their code once per block, so
+// that fetching it (about 200 cycles per 128 bytes that no earlier block has
+// left in the instruction cache) costs more than executing it.
 template <int T>
-__device__ __forceinline__ int block_exclusive_scan(int v, int* warp_sums, int& total)
+__device__ __noinline__ int2 block_exclusive_scan(int v, int* warp_sums)
 {
     constexpr int kWarps = T / 32;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -45,8 +48,8 @@ __device__ __forceinline__ int block_exclusive_scan(int v, int* warp_sums, int& 
         const int y = __shfl_up_sync(0xffffffffu, wi, o);
         if (lane >= o) wi += y;
     }
-    total = __shfl_sync(0xffffffffu, wi, 31);
-    return __shfl_sync(0xffffffffu, wi - w, warp) + incl - v;
+    return make_int2(__shfl_sync(0xffffffffu, wi - w, warp) + incl - v,
+                     __shfl_sync(0xffffffffu, wi, 31));
 }
 
 // x[k] = src[i0 + k] for the thread's PER positions (0 at and past n), with
@@ -74,66 +77,41 @@ __device__ __forceinline__ void load_run(const float* __restrict__ src, int i0, 
 // then the boundary bin is gathered, and its keys (at most kFew, else the
 // range narrows by another histogram) find their own rank: a thread counts
 // the gathered keys above and equal to its own, and the one whose ranks span
-// k publishes the result.  Five block barriers in the usual case.
+// k publishes the result.  Six block barriers in the usual case.
 template <int T>
 struct SelectScratch {
-    // fewer keys need fewer bins, and one warp walks them all
-    static constexpr int kBins = T >= 512 ? 2048 : (T >= 256 ? 1024 : 512);
-    static constexpr int kFew = 256;  // keys that are ranked by counting
+    static constexpr int kBins = 4 * T;  // one 16-byte piece per thread
+    static constexpr int kFew = 256;     // keys that are ranked by counting
     __align__(16) int bins[kBins];
     __align__(16) uint32_t few[kFew];
     uint32_t lo[32], hi[32];  // per-warp key ranges
-    int out[3];               // boundary bin, count above it left over, keys in it
+    int sums[32];
+    int out[3];               // boundary bin, how many of its keys are taken, its keys
     uint32_t tau;
     int need, eq;
     int nfew;
 };
 
-// By one warp: the highest bin from which the count from the top reaches
-// `remaining`; out = {bin, how many of its keys are taken, its keys}.
-template <int BINS>
-__device__ __forceinline__ void boundary_bin(const int* bins, int remaining, int* out)
+// The highest bin from which the count from the top reaches `remaining`, into
+// sc.out: thread t holds four bins, the highest first, and the counts above
+// them come from a block scan.  Two block barriers.
+template <int T>
+__device__ __forceinline__ void boundary_bin(SelectScratch<T>& sc, int remaining)
 {
-    constexpr int BL = BINS / 32;  // bins per lane
-    static_assert(BL == 64 || BL == 32 || BL == 16, "two, one or half a bin per lane below");
-    const int lane = threadIdx.x & 31;
-    const int4* b4 = reinterpret_cast<const int4*>(bins) + (BL / 4) * lane;
-    int mine = 0;
-#pragma unroll
-    for (int q = 0; q < BL / 4; ++q) {
-        const int4 v = b4[(q + lane) & (BL / 4 - 1)];
-        mine += v.x + v.y + v.z + v.w;
+    const int piece = T - 1 - (int)threadIdx.x;
+    const int4 c = reinterpret_cast<const int4*>(sc.bins)[piece];
+    const int mine = c.x + c.y + c.z + c.w;
+    int left = remaining - block_exclusive_scan<T>(mine, sc.sums).x;
+    if (left > 0 && left <= mine) {
+        int bin = 4 * piece + 3, n = c.w;
+        if (left > n) { left -= n; n = c.z; --bin; }
+        if (bin == 4 * piece + 2 && left > n) { left -= n; n = c.y; --bin; }
+        if (bin == 4 * piece + 1 && left > n) { left -= n; n = c.x; --bin; }
+        sc.out[0] = bin;
+        sc.out[1] = left;
+        sc.out[2] = n;
     }
-    int incl = mine;  // keys in this lane's bins and above
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const int y = __shfl_down_sync(0xffffffffu, incl, o);
-        if (lane + o < 32) incl += y;
-    }
-    const uint32_t hit = __ballot_sync(0xffffffffu, incl >= remaining);
-    const int lb = hit ? 31 - __clz(hit) : 0;
-    const int above = __shfl_sync(0xffffffffu, incl - mine, lb);
-    // the boundary lane's bins: two, one or (below 32) at most one per lane
-    constexpr int PL = BL == 64 ? 2 : 1;
-    const int b0 = BL * lb + PL * lane;
-    const bool held = PL * lane < BL;
-    const int c0 = held ? bins[b0] : 0, c1 = (PL == 2) ? bins[b0 + 1] : 0;
-    const int pair = c0 + c1;
-    int inc2 = pair;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const int y = __shfl_down_sync(0xffffffffu, inc2, o);
-        if (lane + o < 32) inc2 += y;
-    }
-    const uint32_t hit2 = __ballot_sync(0xffffffffu, held && above + inc2 >= remaining);
-    const int l2 = hit2 ? 31 - __clz(hit2) : 0;
-    if (lane == l2) {
-        const int before = above + inc2 - pair;  // keys above this lane's bins
-        const bool top = PL == 2 && before + c1 >= remaining;
-        out[0] = top ? b0 + 1 : b0;
-        out[1] = (PL == 1 || top) ? remaining - before : remaining - before - c1;
-        out[2] = top ? c1 : c0;
-    }
+    __syncthreads();
 }
 
 // each(f) calls f(included, key) for every element of the calling thread
@@ -170,8 +148,7 @@ __device__ __forceinline__ SelectResult select_each(EachFn each, int k, SelectSc
             if (in && d <= last) atomicAdd(&sc.bins[d >> shift], 1);
         });
         __syncthreads();
-        if (warp == 0) boundary_bin<S::kBins>(sc.bins, remaining, sc.out);
-        __syncthreads();
+        boundary_bin<T>(sc, remaining);
         lo += (uint32_t)sc.out[0] << shift;
         remaining = sc.out[1];
         const int in_bin = sc.out[2];
