@@ -28,7 +28,9 @@
 // the (unit, 128-token tile) space.  The epilogue groups meet
 // through shared-memory slots and arrival counters, never at a barrier.
 // The epilogues are bound by instruction issue, so the common plans are
-// compiled with their job counts, job sizes and window as constants.
+// compiled with their job counts, job sizes and window as constants (the two
+// passes of 256 units x 3001 tokens with 128 rows, one job per tile: 92 us
+// counted at run time, 80 compiled).
 // Every wait is bounded: on timeout the CTA raises an abort flag, records
 // kErrTimeout in the error word, drains its own copies and MMAs, frees TMEM
 // and returns.
@@ -1224,6 +1226,10 @@ __global__ void __launch_bounds__(kThreads, 1) window_tc_kernel(TcArgs a, Plan p
                 epilogue_stats<D, 4, true>(a, L, sm, b, pl.q_rows, pl.last_m64);
             else if (nrb == 2 && !pl.last_m64)
                 epilogue_stats<D, 2, false>(a, L, sm, b, pl.q_rows, pl.last_m64);
+            else if (nrb == 1 && !pl.last_m64)
+                epilogue_stats<D, 1, false>(a, L, sm, b, pl.q_rows, pl.last_m64);
+            else if (nrb == 1)
+                epilogue_stats<D, 1, true>(a, L, sm, b, pl.q_rows, pl.last_m64);
             else
                 epilogue_stats<D, 0, false>(a, L, sm, b, pl.q_rows, pl.last_m64);
         }
@@ -1242,8 +1248,16 @@ __global__ void __launch_bounds__(kThreads, 1) window_tc_kernel(TcArgs a, Plan p
                 epilogue_scores<D, true, 1, 1, 0>(a, pl, L, sm, b, jt);
             else
                 epilogue_scores<D, true, 1, 0, 0>(a, pl, L, sm, b, jt);
-        } else if (a.s.W % 16 == 0)
-            epilogue_scores<D, true, 2, 0, 0>(a, pl, L, sm, b, jt);
+        } else if (a.s.W % 16 == 0) {
+            if (pl.n_jobs == 1 && pl.granules == 8 && a.s.W == 32)
+                epilogue_scores<D, true, 2, 1, 8, 32>(a, pl, L, sm, b, jt);
+            else if (pl.n_jobs == 1 && pl.granules == 8)
+                epilogue_scores<D, true, 2, 1, 8>(a, pl, L, sm, b, jt);
+            else if (pl.n_jobs == 1)
+                epilogue_scores<D, true, 2, 1, 0>(a, pl, L, sm, b, jt);
+            else
+                epilogue_scores<D, true, 2, 0, 0>(a, pl, L, sm, b, jt);
+        }
         else  // W % 16 != 0: always four accumulators (see launch_impl)
             epilogue_scores<D, false, 2, 0, 0>(a, pl, L, sm, b, jt);
     }
@@ -1314,8 +1328,9 @@ cudaError_t launch_impl(const TcArgs& args, const TcMaps& m, cudaStream_t st)
     }
     Smem L;
     bool fits = false;
-    // (a window that is not a multiple of 16 rows always takes 128-row jobs)
-    for (int attempt = a.s.W % 16 == 0 ? 0 : 1; attempt < 2 && !fits; ++attempt) {
+    // (a window that is not a multiple of 16 rows always takes 128-row jobs, and
+    // up to 128 rows are one such job: four accumulators instead of two)
+    for (int attempt = a.s.W % 16 == 0 && granules > 8 ? 0 : 1; attempt < 2 && !fits; ++attempt) {
         const int per_job = PASS == 1 ? 8 : (attempt == 0 ? 16 : 8);  // granules
         pl.n_jobs = PASS == 1 ? (pl.by_block ? 1 : pl.blocks) : (granules + per_job - 1) / per_job;
         pl.granules = PASS == 1 ? 8 * pl.n_jobs : granules;
