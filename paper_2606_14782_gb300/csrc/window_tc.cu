@@ -30,7 +30,8 @@
 // The epilogues are bound by instruction issue, so the common plans are
 // compiled with their job counts, job sizes and window as constants (the two
 // passes of 256 units x 3001 tokens with 128 rows, one job per tile: 92 us
-// counted at run time, 80 compiled).
+// counted at run time, 80 compiled; steps with 192, 256 and 384 rows 4, 2 and
+// 5 %).
 // Every wait is bounded: on timeout the CTA raises an abort flag, records
 // kErrTimeout in the error word, drains its own copies and MMAs, frees TMEM
 // and returns.
@@ -1226,6 +1227,12 @@ __global__ void __launch_bounds__(kThreads, 1) window_tc_kernel(TcArgs a, Plan p
                 epilogue_stats<D, 4, true>(a, L, sm, b, pl.q_rows, pl.last_m64);
             else if (nrb == 2 && !pl.last_m64)
                 epilogue_stats<D, 2, false>(a, L, sm, b, pl.q_rows, pl.last_m64);
+            else if (nrb == 2)
+                epilogue_stats<D, 2, true>(a, L, sm, b, pl.q_rows, pl.last_m64);
+            else if (nrb == 3 && !pl.last_m64)
+                epilogue_stats<D, 3, false>(a, L, sm, b, pl.q_rows, pl.last_m64);
+            else if (nrb == 4)
+                epilogue_stats<D, 4, false>(a, L, sm, b, pl.q_rows, pl.last_m64);
             else if (nrb == 1 && !pl.last_m64)
                 epilogue_stats<D, 1, false>(a, L, sm, b, pl.q_rows, pl.last_m64);
             else if (nrb == 1)
@@ -1238,12 +1245,18 @@ __global__ void __launch_bounds__(kThreads, 1) window_tc_kernel(TcArgs a, Plan p
                 epilogue_scores<D, true, 1, 2, 14, 64>(a, pl, L, sm, b, jt);
             else if (pl.n_jobs == 2 && pl.granules == 28)
                 epilogue_scores<D, true, 1, 2, 14>(a, pl, L, sm, b, jt);
+            else if (pl.n_jobs == 2 && pl.granules == 24)
+                epilogue_scores<D, true, 1, 2, 12>(a, pl, L, sm, b, jt);
             else if (pl.n_jobs == 2)
                 epilogue_scores<D, true, 1, 2, 0>(a, pl, L, sm, b, jt);
             else if (pl.n_jobs == 1 && pl.granules == 14 && a.s.W == 32)
                 epilogue_scores<D, true, 1, 1, 14, 32>(a, pl, L, sm, b, jt);
             else if (pl.n_jobs == 1 && pl.granules == 14)
                 epilogue_scores<D, true, 1, 1, 14>(a, pl, L, sm, b, jt);
+            else if (pl.n_jobs == 1 && pl.granules == 16)
+                epilogue_scores<D, true, 1, 1, 16>(a, pl, L, sm, b, jt);
+            else if (pl.n_jobs == 1 && pl.granules == 12)
+                epilogue_scores<D, true, 1, 1, 12>(a, pl, L, sm, b, jt);
             else if (pl.n_jobs == 1)
                 epilogue_scores<D, true, 1, 1, 0>(a, pl, L, sm, b, jt);
             else
