@@ -125,8 +125,8 @@ __device__ __forceinline__ int ties_before(const float* x, int nv, const SelectR
     return block_exclusive_scan<T>(eq, warp_sums).x;
 }
 
-// The residual E of the thread's run into x (0 at and past N), added to v
-// when use_E, and the coherence (Eqs. 5-7) with the radius R a constant:
+// The residual E of the thread's run (x, 0 at and past N), added to v when
+// use_E, and the coherence (Eqs. 5-7) with the radius R a constant:
 // v[k] += the mean of E over [i - R, i + R] clipped to [0, N), for the run's
 // positions i = i0 + k < N.  The R values on either side come from the
 // neighbouring lanes' runs by shuffles (from global memory at a warp's two
@@ -135,11 +135,10 @@ __device__ __forceinline__ int ties_before(const float* x, int nv, const SelectR
 // R <= PER and every lane of the warp.
 template <int PER, int R>
 __device__ __forceinline__ void coherence_run(const float* __restrict__ Ec, int i0, int N,
-                                              bool use_E, float* x, float* v)
+                                              bool use_E, const float* x, float* v)
 {
     static_assert(R <= PER, "the halo must come from the adjacent run");
     const int lane = threadIdx.x & 31;
-    load_run<PER>(Ec, i0, N, x);
     float gl[R], gh[R];
 #pragma unroll
     for (int m = 0; m < R; ++m) {
@@ -216,7 +215,7 @@ __host__ __device__ constexpr bool run_fits(int PER, int R) { return R <= PER &&
 // 7, 9) compiled as constants where the registers allow.
 template <int PER>
 __device__ __forceinline__ void residual_and_coherence(const float* __restrict__ Ec, int i0, int N,
-                                                       int r, bool use_E, float* x, float* v)
+                                                       int r, bool use_E, const float* x, float* v)
 {
     if constexpr (run_fits(PER, 3))
         if (r == 3) return coherence_run<PER, 3>(Ec, i0, N, use_E, x, v);
@@ -226,7 +225,6 @@ __device__ __forceinline__ void residual_and_coherence(const float* __restrict__
         if (r == 7) return coherence_run<PER, 7>(Ec, i0, N, use_E, x, v);
     if constexpr (run_fits(PER, 9))
         if (r == 9) return coherence_run<PER, 9>(Ec, i0, N, use_E, x, v);
-    load_run<PER>(Ec, i0, N, x);
     if (use_E) {
 #pragma unroll
         for (int k = 0; k < PER; ++k) v[k] += x[k];
@@ -286,12 +284,13 @@ __device__ __forceinline__ void add_layers(const Residuals& E, int l0, int n, in
 }
 
 // The evidence V = E + L + T of the thread's run (Eqs. 5-11) into v, 0 at and
-// past N; x is scratch for PER floats.
+// past N; x: the run of the layer's own residuals, at Ec (runs of 8: loaded
+// by the caller, ahead of the layers before).
 template <int PER>
 __device__ __forceinline__ void evidence_run(const Calib& c, const Residuals& E, int layer, int i0,
-                                             int N, float* x, float* v)
+                                             int N, const float* __restrict__ Ec, float* x,
+                                             float* v)
 {
-    const float* Ec = E.row(layer);
 #pragma unroll
     for (int k = 0; k < PER; ++k) v[k] = 0.f;
     // persistence: mean of E over the preceding min(m, l) layers (Eqs. 8-9)
@@ -303,10 +302,10 @@ __device__ __forceinline__ void evidence_run(const Calib& c, const Residuals& E,
         for (int k = 0; k < PER; ++k) v[k] *= inv_prev;
     }
     // E, and the coherence: truncated radius-r box mean of E (Eqs. 5-7)
+    if (PER > 8) load_run<PER>(Ec, i0, N, x);
     if (c.use_L) {
         residual_and_coherence<PER>(Ec, i0, N, c.r, c.use_E, x, v);
     } else if (c.use_E) {
-        load_run<PER>(Ec, i0, N, x);
 #pragma unroll
         for (int k = 0; k < PER; ++k) v[k] += x[k];
     }
@@ -461,17 +460,23 @@ __device__ __forceinline__ void calibrate_unit(const Shape& s, const Calib& c, c
     uint32_t kmin = 0xffffffffu, kmax = 0u;  // range of b's keys over the candidates
     int M = 0;
     if (a.compute_scores) {
+        // (runs of 8: B, the residuals and then the layers before are in
+        // flight together)
+        const float* Bu = a.B + (size_t)u * N;
+        if (!kPark) load_run<PER>(Bu, i0, N, b);
         {
             float x[PER];
-            evidence_run<PER>(c, residuals_of(a, s, rq, h), layer, i0, N, x, v);
+            const Residuals E = residuals_of(a, s, rq, h);
+            const float* Ec = E.row(layer);
+            if (!kPark) load_run<PER>(Ec, i0, N, x);
+            evidence_run<PER>(c, E, layer, i0, N, Ec, x, v);
         }
         if (a.V) store_run<PER>(a.V + (size_t)u * N, i0, N, v);
         if (kPark) {
 #pragma unroll
             for (int k = 0; k < PER; ++k) sm[k * T + threadIdx.x] = v[k];
         }
-        const float* Bu = a.B + (size_t)u * N;
-        load_run<PER>(Bu, i0, N, b);
+        if (kPark) load_run<PER>(Bu, i0, N, b);
         pool_run<PER>(Bu, i0, n_cand, c.pool / 2, b, kmin, kmax);
         if (a.Bp) store_run<PER>(a.Bp + (size_t)u * N, i0, N, b);
         M = match_count(c.rho, a.calib_budget[pair], N, win, n_cand);
@@ -652,8 +657,14 @@ calibrate_sweep_kernel(Shape s, CalibTable t, SweepArgs sw, CalibArgs a)
             if (i0 + 8 * q < n_cand) mem |= (uint32_t)map[i0 / 8 + q] << (8 * q);
     }
     float x[PER], v[PER], b[PER];
-    evidence_run<PER>(c, residuals_of(a, s, rq, h), layer, i0, N, x, v);
-    load_run<PER>(sw.pooled + (size_t)u * N, i0, N, b);
+    const Residuals E = residuals_of(a, s, rq, h);
+    const float* Ec = E.row(layer);
+    if (PER <= 8) {
+        load_run<PER>(sw.pooled + (size_t)u * N, i0, N, b);
+        load_run<PER>(Ec, i0, N, x);
+    }
+    evidence_run<PER>(c, E, layer, i0, N, Ec, x, v);
+    if (PER > 8) load_run<PER>(sw.pooled + (size_t)u * N, i0, N, b);
     float lam = 0.f;
     if (M > 0) {
         float sv[1] = {0.f};
