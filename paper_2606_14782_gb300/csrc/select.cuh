@@ -152,7 +152,7 @@ __device__ __forceinline__ SelectResult select_each(EachFn each, int k, SelectSc
         lo += (uint32_t)sc.out[0] << shift;
         remaining = sc.out[1];
         const int in_bin = sc.out[2];
-        last = (1u << shift) - 1u;
+        last = min((1u << shift) - 1u, ~lo);  // (the top bin may reach past 2^32)
         if (shift == 0) return {lo, remaining, in_bin};
         if (in_bin <= S::kFew) break;
         // many keys in one bin (plateaus of equal scores): narrow the range
