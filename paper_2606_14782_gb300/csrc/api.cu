@@ -46,7 +46,7 @@ bacon_status cuda_fail(cudaError_t e, const char* what)
 bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
 constexpr int kChunkTokens = 1024;  // pass-1 token chunk (multiple of the 128-token tile)
-constexpr size_t kLastBytes = 16ull << 20;  // host path: keys of the last pipelined part, at most
+constexpr size_t kLastBytes = 24ull << 20;  // host path: keys of the last pipelined part, at most
 constexpr int kMaxSeq = 24576;      // calibration keeps 2 x N fp32 in shared memory
 static_assert(kMaxVariants == BACON_MAX_VARIANTS, "variant table size");
 
@@ -1095,10 +1095,12 @@ bacon_status bacon_compress_host(bacon_ctx* ctx, int requests, const void* q_win
     // part computes.  A part is a whole request, except that the last request
     // is halved again and again: only what follows the last upload is not
     // hidden behind the link, one small part's compression and download.
-    // (Every further part costs about 12 us of copy and kernel overheads, so
-    // the halving ends at kLastBytes of keys.)  28 layers x 4096 tokens, one
-    // request: 968 us whole, 826 halved; equal parts of 32, 16 and 8 MB of
-    // keys took 851, 895 and 1038 us.
+    // (A part's dependent launches take some 75 us, as long as 14 MB take on
+    // the link, so the halving ends at kLastBytes of keys: below that the
+    // parts queue behind one another.  11 layers of 3.8 MB: 393 us whole, 334
+    // in two parts, 401 in three.)  28 layers x 4096 tokens, one request: 968
+    // us whole, 805 halved; equal parts of 32, 16 and 8 MB took 851, 895 and
+    // 1038 us.
     const int L = ctx->layers;
     struct Part {
         int r, l0, n;

@@ -41,10 +41,10 @@ using namespace sel;
 
 // Threads per CTA and positions per thread depend on the prompt length only
 // (so that every call on the same shape reduces in the same order and gives
-// the same bits), sized so that threads x positions stays close to N: 8 positions per thread on 128, 256,
-// 512 or 1024 threads up to 1024, 2048, 4096 or 8192 tokens (several CTAs
-// share an SM below 1024 threads), then 1024 threads of 16 positions up to
-// 16384 tokens and of 24 up to 24576.
+// the same bits), sized so that threads x positions stays close to N: 8
+// positions per thread on 128, 256, 512 or 1024 threads up to 1024, 2048,
+// 4096 or 8192 tokens (several CTAs share an SM below 1024 threads), then
+// 1024 threads of 16 positions up to 16384 tokens and of 24 up to 24576.
 constexpr int kMaxPrompt = 24576;
 
 // Block-wide fp32 sums of NV values in one round, by a shuffle tree (pairwise,
