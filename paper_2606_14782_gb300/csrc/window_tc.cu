@@ -280,6 +280,13 @@ __device__ __forceinline__ void write_bias_row(uint8_t* bias, const JobTable& jt
     *reinterpret_cast<uint32_t*>(bias + off + 4) = (uint32_t)__bfloat16_as_ushort(lo);
 }
 
+// Zeros in one slot of the bias operand, by `threads` threads.
+__device__ __forceinline__ void zero_bias(uint8_t* bias, int bias_rows, int thread, int threads)
+{
+    for (int i = thread; i < bias_rows * 8; i += threads)
+        reinterpret_cast<uint4*>(bias)[i] = make_uint4(0u, 0u, 0u, 0u);
+}
+
 // The bias operand of unit u, by the 32 lanes of the producer warp (the
 // normalisers of a lane's rows are loaded eight at a time).
 __device__ __forceinline__ void write_bias(const TcArgs& a, uint8_t* bias, int u, const JobTable& jt,
@@ -310,8 +317,15 @@ __device__ __forceinline__ void write_bias(const TcArgs& a, uint8_t* bias, int u
 
 // All 32 lanes run the loop; lane 0 issues the copies.  At each new unit the
 // window rows are reloaded once the previous unit's MMAs have released them
-// (pass 2 also rewrites the bias operand, a second arrival on q_full; the
-// CTA's first unit has its bias from the kernel's prologue).
+// (pass 2 also rewrites the bias operand, a second arrival on q_full).
+//
+// Who writes a slot's bias: the producer runs while the other warps still set
+// up, so the prologue touches slot 0 alone (its zeros and the first unit's
+// values), which the producer writes again only once q_empty(0) has come back
+// from MMAs issued after the prologue's barrier.  Slot 1 starts free, nothing
+// orders the producer's first use of it after the prologue, and so it is the
+// producer's from the start, zeros included (bias_rows / 4 stores a lane,
+// once per CTA, and only when its range reaches a second unit).
 template <int D, int PASS>
 __device__ __forceinline__ void produce(const TcArgs& a, const TcMaps& maps, const Plan& pl,
                                         const Smem& L, uint8_t* sm, const Bars& b,
@@ -353,7 +367,12 @@ __device__ __forceinline__ void produce(const TcArgs& a, const TcMaps& maps, con
             }
             if (PASS == 2) {
                 if (qloads > 0) {
-                    write_bias(a, sm + L.bias + slot * L.bias_slot, u, jt, pl.granules, inv_c);
+                    uint8_t* bias = sm + L.bias + slot * L.bias_slot;
+                    if (qloads < q_slots) {  // slot 1 for the first time
+                        zero_bias(bias, pl.bias_rows, lane, 32);
+                        __syncwarp();
+                    }
+                    write_bias(a, bias, u, jt, pl.granules, inv_c);
                     tc::fence_proxy_async_smem();
                     __syncwarp();
                 }
@@ -1200,15 +1219,15 @@ __global__ void __launch_bounds__(kThreads, 1) window_tc_kernel(TcArgs a, Plan p
     if (warp != 0) after_previous();
     if (PASS == 2 && warp >= 2) {
         // constant operand: 1 in columns 0-2 of every token row (one atom of
-        // 8 rows when ones_atom); the bias operand starts zeroed, then takes
-        // the first unit's values (the producer rewrites it for later units)
+        // 8 rows when ones_atom); slot 0 of the bias operand starts zeroed,
+        // then takes the first unit's values (later units' and slot 1 are the
+        // producer's, see there)
         const int row = threadIdx.x - 64;
         int g0, g1;
         item_range(a.items, &g0, &g1);
         const int u = g0 / ((a.s.N + kTileTok - 1) / kTileTok);
         const float x = row < 16 * pl.granules ? row_bias(a, u, row, sqrtf((float)D) / kLog2e) : 0.f;
-        for (int i = row; i < pl.q_slots * pl.bias_rows * 8; i += kEpiThreads)
-            reinterpret_cast<uint4*>(sm + L.bias)[i] = make_uint4(0u, 0u, 0u, 0u);
+        zero_bias(sm + L.bias, pl.bias_rows, row, kEpiThreads);
         if (row < (pl.ones_atom ? 8 : 128)) {
             uint4* ones = reinterpret_cast<uint4*>(sm + L.ones + row * 128);
             for (int q = 0; q < 8; ++q) ones[q] = make_uint4(0u, 0u, 0u, 0u);

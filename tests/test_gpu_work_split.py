@@ -61,6 +61,63 @@ def test_few_units_and_many_give_the_same_bits(group, window, head_dim, seq_len)
     ctx.close()
 
 
+def _window_scores(q, k, window):
+    """B, Q, E of one layer, q [Hq, W, d] and k [Hkv, N, d], without a context."""
+    hkv, n, d = k.shape
+    out = torch.empty(3, hkv, n, device="cuda")
+    rc = bacon.load().bacon_window_scores_noalloc(
+        hkv, q.shape[0], d, window, q.data_ptr(), k.data_ptr(), n, *(t.data_ptr() for t in out),
+        torch.cuda.current_stream().cuda_stream)
+    assert rc == bacon.BACON_OK
+    return out
+
+
+# Window rows that leave pass 2 two slots of them (and of their bias) in shared
+# memory, and more tiles than SMs, so that a CTA's share ends one unit after
+# one to a few tiles and goes on with the next.  A kv-head by itself has fewer
+# tiles than there are SMs: every CTA then works on one tile of one unit.
+@pytest.mark.parametrize("hkv,group,window,head_dim,seq_len", [
+    (32, 1, 32, 128, 3000),
+    (128, 1, 32, 128, 129),
+    (128, 1, 32, 64, 257),
+    (128, 1, 32, 128, 500),
+    (32, 4, 32, 128, 700),
+    (16, 2, 64, 128, 1537),
+    (12, 4, 32, 64, 2049),
+    (16, 4, 64, 64, 1500),
+    (20, 5, 13, 128, 1100),  # any window
+])
+def test_shares_that_cross_short_units(hkv, group, window, head_dim, seq_len):
+    g = torch.Generator(device="cuda").manual_seed(hkv * seq_len)
+    q, k = (torch.randn(*shape, generator=g, device="cuda").to(torch.bfloat16)
+            for shape in ((hkv * group, window, head_dim), (hkv, seq_len, head_dim)))
+    got = _window_scores(q, k, window)
+    for h in range(hkv):
+        alone = _window_scores(q[h * group:(h + 1) * group], k[h:h + 1], window)
+        assert torch.equal(got[:, h], alone[:, 0]), h
+
+
+def test_whole_step_shares_that_cross_units():
+    """The same with the normalisers from a launch of their own."""
+    layers, requests, hkv, group, window, d, n = 6, 2, 8, 4, 32, 128, 700
+    wl = workloads.CONFIGS["tiny"].with_(
+        layers=layers, requests=requests, q_heads=group * hkv, kv_heads=hkv, head_dim=d,
+        seq_len=n, window=window, visual=(16, n - 100))
+    x = workloads.generate(wl, seed=13, device="cuda")
+    ctx = bacon.Context(layers, hkv, group * hkv, d, window, 7, 100, max_seq_len=n,
+                        max_requests=requests)
+    ctx.compress_all_layers(x.qwin, x.k, x.v, 100)
+    got = torch.stack([ctx.scores(s) for s in "BQE"]).view(3, requests, layers, hkv, n)
+    ctx.sync()
+    for r in range(requests):
+        for l in range(layers):
+            for h in range(hkv):
+                alone = _window_scores(x.qwin[r, l, h * group:(h + 1) * group],
+                                       x.k[r, l, h:h + 1], window)
+                assert torch.equal(got[:, r, l, h], alone[:, 0]), (r, l, h)
+    ctx.close()
+
+
 @pytest.mark.parametrize("offset", [0, 1, 2, 4])
 def test_scores_out_at_any_float_alignment(offset):
     """Aligned score rows are stored by the kernel, others copied: same bits."""

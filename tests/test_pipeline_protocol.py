@@ -53,8 +53,13 @@ def wait(bar, k):
         raise Fault(f"{bar.name}: waited for phase {k}, barrier at phase {bar.phase}")
 
 
-def simulate(chunks, n_tiles, tpc, jobs_per_tile, nbuf, stages, q_slots, pass2, guard, seed):
-    """chunks: the CTA's list of (unit, chunk index); n_tiles: tiles per unit."""
+def simulate(chunks, n_tiles, tpc, jobs_per_tile, nbuf, stages, q_slots, pass2, guard, seed,
+             prologue_slots=1):
+    """chunks: the CTA's list of (unit, chunk index); n_tiles: tiles per unit.
+    The producer starts before the CTA is set up; the MMA thread and the
+    epilogue wait for the set-up.  In pass 2 the set-up zeroes the first
+    `prologue_slots` slots of the bias operand and fills slot 0 for the first
+    unit; the producer zeroes the other slot itself and writes later units'."""
     rnd = random.Random(seed)
     t_full = [Bar(1, f"t_full{i}") for i in range(nbuf)]
     t_empty = [Bar(16, f"t_empty{i}") for i in range(nbuf)]
@@ -68,8 +73,25 @@ def simulate(chunks, n_tiles, tpc, jobs_per_tile, nbuf, stages, q_slots, pass2, 
     tma = []       # pending TMA completions (any order)
     commits = []   # pending MMA-commit arrivals (in issue order)
 
+    ready = []     # set up
+    bias = [None] * q_slots  # whose bias a slot holds
+
     def tiles_of(ci):
         return range(ci * tpc, min(n_tiles, (ci + 1) * tpc))
+
+    def setup():
+        if pass2:
+            for slot in range(min(prologue_slots, q_slots)):
+                yield
+                bias[slot] = "zeros"
+            yield
+            bias[0] = chunks[0][0]
+        yield
+        ready.append(True)
+
+    def wait_ready():
+        while not ready:
+            yield
 
     def producer():
         cur, qloads, kt = -1, 0, 0
@@ -80,6 +102,12 @@ def simulate(chunks, n_tiles, tpc, jobs_per_tile, nbuf, stages, q_slots, pass2, 
                 tma.append(q_full[slot])
                 if pass2:
                     yield
+                    if qloads > 0:
+                        if qloads < q_slots:
+                            bias[slot] = "zeros"
+                            yield
+                        bias[slot] = u
+                        yield
                     q_full[slot].arrive()
                 qloads += 1
                 cur = u
@@ -98,6 +126,7 @@ def simulate(chunks, n_tiles, tpc, jobs_per_tile, nbuf, stages, q_slots, pass2, 
 
     def mma():
         cur, cur_slot, qwaits, kt, job = -1, 0, 0, 0, 0
+        yield from wait_ready()
         for u, ci in chunks:
             if u != cur:
                 if cur >= 0:
@@ -114,6 +143,8 @@ def simulate(chunks, n_tiles, tpc, jobs_per_tile, nbuf, stages, q_slots, pass2, 
                     buf, nb = job % nbuf, job // nbuf
                     job += 1
                     yield from wait(t_empty[buf], nb - 1)
+                    if pass2 and bias[cur_slot] != u:
+                        raise Fault(f"unit {u}'s MMAs read the bias of {bias[cur_slot]}")
                     commits.append(t_full[buf])
                     yield
                 commits.append(k_empty[st])
@@ -122,6 +153,7 @@ def simulate(chunks, n_tiles, tpc, jobs_per_tile, nbuf, stages, q_slots, pass2, 
 
     def epilogue(q, g):
         job = n = 0
+        yield from wait_ready()
         for u, ci in chunks:
             ts = list(tiles_of(ci))
             for i, _ in enumerate(ts):
@@ -147,7 +179,7 @@ def simulate(chunks, n_tiles, tpc, jobs_per_tile, nbuf, stages, q_slots, pass2, 
                     yield
                     x_empty[(par, q)].arrive()
 
-    procs = [producer(), mma()] + [epilogue(q, g) for q in range(4) for g in range(4)]
+    procs = [producer(), mma(), setup()] + [epilogue(q, g) for q in range(4) for g in range(4)]
     live = list(range(len(procs)))
     for _ in range(500000):
         if not live and not tma and not commits:
@@ -209,6 +241,23 @@ def test_model_catches_the_unguarded_merger():
     # x_full wait passes on the slot's previous phase
     chunks = cta_range(3, 2, 1, 0)
     faults = [simulate(chunks, 11, 8, 1, 4, 4, 1, True, False, s) for s in range(8)]
+    assert any(f is not None for f in faults)
+
+
+# units of one to four tiles, of which a CTA takes several: its producer is at
+# the second unit's bias while the CTA may still be setting up
+@pytest.mark.parametrize("n_tiles", [1, 2, 3, 4])
+@pytest.mark.parametrize("q_slots", [1, 2])
+def test_bias_slots_of_short_units(n_tiles, q_slots):
+    for seed in range(12):
+        fault = simulate(cta_range(5, 1, 1, 0), n_tiles, 8, 1, 4, 4, q_slots, True, True, seed)
+        assert fault is None, (seed, fault)
+
+
+def test_model_catches_a_prologue_that_zeroes_both_slots():
+    chunks = cta_range(5, 1, 1, 0)
+    faults = [simulate(chunks, 1, 8, 1, 4, 4, 2, True, True, s, prologue_slots=2)
+              for s in range(12)]
     assert any(f is not None for f in faults)
 
 
