@@ -64,12 +64,12 @@ def test_few_units_and_many_give_the_same_bits(group, window, head_dim, seq_len)
 def _window_scores(q, k, window):
     """B, Q, E of one layer, q [Hq, W, d] and k [Hkv, N, d], without a context."""
     hkv, n, d = k.shape
-    out = torch.empty(3, hkv, n, device="cuda")
+    out = [torch.empty(hkv, n, device="cuda") for _ in range(3)]  # each 16-byte aligned
     rc = bacon.load().bacon_window_scores_noalloc(
         hkv, q.shape[0], d, window, q.data_ptr(), k.data_ptr(), n, *(t.data_ptr() for t in out),
         torch.cuda.current_stream().cuda_stream)
     assert rc == bacon.BACON_OK
-    return out
+    return torch.stack(out)
 
 
 # Window rows that leave pass 2 two slots of them (and of their bias) in shared
