@@ -142,8 +142,7 @@ adaptive_select_kernel(Shape s, int keep_window, AdaptArgs a)
 // Flat per-layer gather: output row j of a pair belongs to the head whose
 // segment (per-head counts, heads in order) contains it.
 __global__ void __launch_bounds__(256)
-gather_flat_kernel(GatherTable tab, Shape s, const int32_t* __restrict__ counts,
-                   int* __restrict__ err)
+gather_flat_kernel(GatherTable tab, Shape s, const int32_t* counts, int* err)
 {
     after_previous();
     const int pair = blockIdx.y;
@@ -164,8 +163,8 @@ gather_flat_kernel(GatherTable tab, Shape s, const int32_t* __restrict__ counts,
     }
     const size_t in_off = ((size_t)h * s.N + src) * s.d;
     const size_t out_off = (size_t)j * s.d;
-    const uint4 kv = __ldg(reinterpret_cast<const uint4*>(tab.k[pair] + in_off) + q);
-    const uint4 vv = __ldg(reinterpret_cast<const uint4*>(tab.v[pair] + in_off) + q);
+    const uint4 kv = load_input(tab.k[pair] + in_off, q);
+    const uint4 vv = load_input(tab.v[pair] + in_off, q);
     reinterpret_cast<uint4*>(tab.ko[pair] + out_off)[q] = kv;
     reinterpret_cast<uint4*>(tab.vo[pair] + out_off)[q] = vv;
 }

@@ -133,7 +133,7 @@ __device__ __forceinline__ int ties_before(const float* x, int nv, const SelectR
 // window sum slides along the run: drop i - R, add i + 1 + R.  Needs
 // R <= PER and every lane of the warp.
 template <int PER, int R>
-__device__ __forceinline__ void coherence_run(const float* __restrict__ Ec, int i0, int N,
+__device__ __forceinline__ void coherence_run(const float* Ec, int i0, int N,
                                               bool use_E, const float* x, float* v)
 {
     static_assert(R <= PER, "the halo must come from the adjacent run");
@@ -142,8 +142,8 @@ __device__ __forceinline__ void coherence_run(const float* __restrict__ Ec, int 
 #pragma unroll
     for (int m = 0; m < R; ++m) {
         const int jl = i0 - R + m, jh = i0 + PER + m;
-        gl[m] = (lane == 0 && jl >= 0 && jl < N) ? __ldg(Ec + jl) : 0.f;
-        gh[m] = (lane == 31 && jh < N) ? __ldg(Ec + jh) : 0.f;
+        gl[m] = (lane == 0 && jl >= 0 && jl < N) ? Ec[jl] : 0.f;
+        gh[m] = (lane == 31 && jh < N) ? Ec[jh] : 0.f;
     }
     if (use_E) {
 #pragma unroll
@@ -185,21 +185,21 @@ __device__ __forceinline__ void coherence_run(const float* __restrict__ Ec, int 
 
 // The same for any radius, reading the window from global memory (L1).
 template <int PER>
-__device__ __forceinline__ void coherence_any(const float* __restrict__ Ec, int i0, int N, int r,
+__device__ __forceinline__ void coherence_any(const float* Ec, int i0, int N, int r,
                                               float* v)
 {
     const float inv_full = 1.f / (float)(2 * r + 1);
     int lo = max(0, i0 - r), hi = min(N - 1, i0 + r);
     float sum = 0.f;
-    for (int j = lo; j <= hi; ++j) sum += __ldg(Ec + j);
+    for (int j = lo; j <= hi; ++j) sum += Ec[j];
 #pragma unroll
     for (int k = 0; k < PER; ++k) {
         const int i = i0 + k;
         if (i < N) {
             const int cnt = hi - lo + 1;
             v[k] += fmaxf(sum, 0.f) * (cnt == 2 * r + 1 ? inv_full : 1.f / (float)cnt);
-            if (i - r >= 0) sum -= __ldg(Ec + i - r);
-            if (i + 1 + r <= N - 1) sum += __ldg(Ec + i + 1 + r);
+            if (i - r >= 0) sum -= Ec[i - r];
+            if (i + 1 + r <= N - 1) sum += Ec[i + 1 + r];
             lo = max(0, i + 1 - r);
             hi = min(N - 1, i + 1 + r);
         }
@@ -213,7 +213,7 @@ __host__ __device__ constexpr bool run_fits(int PER, int R) { return R <= PER &&
 // E (added to v when use_E) and its coherence, with the paper's radii (3, 5,
 // 7, 9) compiled as constants where the registers allow.
 template <int PER>
-__device__ __forceinline__ void residual_and_coherence(const float* __restrict__ Ec, int i0, int N,
+__device__ __forceinline__ void residual_and_coherence(const float* Ec, int i0, int N,
                                                        int r, bool use_E, const float* x, float* v)
 {
     if constexpr (run_fits(PER, 3))
@@ -262,7 +262,7 @@ __device__ __forceinline__ void add_layers(const Residuals& E, int l0, int n, in
             const float4* p = reinterpret_cast<const float4*>(E.base + slot * E.layer_stride + i0);
 #pragma unroll
             for (int q = 0; q < PER / 4; ++q) {
-                const float4 e = __ldg(p + q);
+                const float4 e = p[q];
                 v[4 * q] += e.x;
                 v[4 * q + 1] += e.y;
                 v[4 * q + 2] += e.z;
@@ -276,7 +276,7 @@ __device__ __forceinline__ void add_layers(const Residuals& E, int l0, int n, in
             const float* p = E.base + slot * E.layer_stride;
 #pragma unroll
             for (int k = 0; k < PER; ++k)
-                if (i0 + k < N) v[k] += __ldg(p + i0 + k);
+                if (i0 + k < N) v[k] += p[i0 + k];
             if (++slot == E.ring) slot = 0;
         }
     }
@@ -287,7 +287,7 @@ __device__ __forceinline__ void add_layers(const Residuals& E, int l0, int n, in
 // by the caller, ahead of the layers before).
 template <int PER>
 __device__ __forceinline__ void evidence_run(const Calib& c, const Residuals& E, int layer, int i0,
-                                             int N, const float* __restrict__ Ec, float* x,
+                                             int N, const float* Ec, float* x,
                                              float* v)
 {
 #pragma unroll
@@ -317,7 +317,7 @@ __device__ __forceinline__ void evidence_run(const Calib& c, const Residuals& E,
 // the candidates, 0 past them) from Bu's run in b, in place; the key range of
 // the candidates goes to kmin, kmax.
 template <int PER>
-__device__ __forceinline__ void pool_run(const float* __restrict__ Bu, int i0, int n_cand, int half,
+__device__ __forceinline__ void pool_run(const float* Bu, int i0, int n_cand, int half,
                                          float* b, uint32_t& kmin, uint32_t& kmax)
 {
     float p[PER];
@@ -331,8 +331,8 @@ __device__ __forceinline__ void pool_run(const float* __restrict__ Bu, int i0, i
 #pragma unroll
         for (int m = 0; m < 3; ++m) {
             const int jl = i0 - 3 + m, jr = i0 + PER + m;
-            hl[m] = (lane == 0 && jl >= 0 && jl < n_cand) ? __ldg(Bu + jl) : -INFINITY;
-            hr[m] = (lane == 31 && jr < n_cand) ? __ldg(Bu + jr) : -INFINITY;
+            hl[m] = (lane == 0 && jl >= 0 && jl < n_cand) ? Bu[jl] : -INFINITY;
+            hr[m] = (lane == 31 && jr < n_cand) ? Bu[jr] : -INFINITY;
         }
 #pragma unroll
         for (int k = 0; k < PER; ++k)
@@ -356,7 +356,7 @@ __device__ __forceinline__ void pool_run(const float* __restrict__ Bu, int i0, i
             p[k] = -INFINITY;
             if (i < n_cand) {
                 const int lo = max(0, i - half), hi = min(n_cand - 1, i + half);
-                for (int v = lo; v <= hi; ++v) p[k] = fmaxf(p[k], __ldg(Bu + v));
+                for (int v = lo; v <= hi; ++v) p[k] = fmaxf(p[k], Bu[v]);
             }
         }
     }

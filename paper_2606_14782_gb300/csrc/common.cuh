@@ -88,6 +88,18 @@ __device__ __forceinline__ void after_previous()
     asm volatile("griddepcontrol.wait;\n griddepcontrol.launch_dependents;\n" ::: "memory");
 }
 
+// Piece q of a row of the caller's K or V through the read-only path: the one
+// place that uses it.  That path is defined for memory which nobody writes
+// while the kernel is resident, and a kernel launched by launch_after is
+// resident while the kernel before it writes, so all that the library's own
+// kernels hand to one another (B, E, S, partial statistics, bitmaps, counts,
+// positions) is read by ordinary loads, through pointers without __restrict__,
+// which after_previous() orders.
+__device__ __forceinline__ uint4 load_input(const uint16_t* row, int q)
+{
+    return __ldg(reinterpret_cast<const uint4*>(row) + q);
+}
+
 template <typename... P, typename... A>
 cudaError_t launch_after(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
                          const A&... args)

@@ -9,7 +9,7 @@ namespace bacon {
 namespace {
 
 __global__ void __launch_bounds__(256)
-gather_kernel(GatherTable tab, Shape s, int* __restrict__ err)
+gather_kernel(GatherTable tab, Shape s, int* err)
 {
     after_previous();
     const int u = blockIdx.y;
@@ -26,12 +26,10 @@ gather_kernel(GatherTable tab, Shape s, int* __restrict__ err)
     }
     const size_t in_off = ((size_t)h * s.N + src) * s.d;
     const size_t out_off = ((size_t)h * kept + j) * s.d;
-    const uint4* ks = reinterpret_cast<const uint4*>(tab.k[pair] + in_off) + q;
-    const uint4* vs = reinterpret_cast<const uint4*>(tab.v[pair] + in_off) + q;
     uint4* kd = reinterpret_cast<uint4*>(tab.ko[pair] + out_off) + q;
     uint4* vd = reinterpret_cast<uint4*>(tab.vo[pair] + out_off) + q;
-    const uint4 kv = __ldg(ks);
-    const uint4 vv = __ldg(vs);
+    const uint4 kv = load_input(tab.k[pair] + in_off, q);
+    const uint4 vv = load_input(tab.v[pair] + in_off, q);
     *kd = kv;
     *vd = vv;
 }

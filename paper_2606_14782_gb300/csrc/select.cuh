@@ -55,13 +55,13 @@ __device__ __noinline__ int2 block_exclusive_scan(int v, int* warp_sums)
 // x[k] = src[i0 + k] for the thread's PER positions (0 at and past n), with
 // 16-byte loads when the run is whole and aligned (n % 4 == 0).
 template <int PER>
-__device__ __forceinline__ void load_run(const float* __restrict__ src, int i0, int n, float* x)
+__device__ __forceinline__ void load_run(const float* src, int i0, int n, float* x)
 {
     if ((n & 3) == 0 && i0 + PER <= n) {
         const float4* s4 = reinterpret_cast<const float4*>(src + i0);
 #pragma unroll
         for (int q = 0; q < PER / 4; ++q) {
-            const float4 v = __ldg(s4 + q);
+            const float4 v = s4[q];
             x[4 * q] = v.x;
             x[4 * q + 1] = v.y;
             x[4 * q + 2] = v.z;

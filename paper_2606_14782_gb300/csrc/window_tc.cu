@@ -235,7 +235,7 @@ __device__ __forceinline__ uint32_t sw128_offset(int row, int col)
 // log2 of one window row's softmax normaliser over all chunks, plus
 // log2(G W), so that pass 2's 2^(logit' - lse2) is A_{q,i} / (G W).  p: the
 // row's partials, `rows` apart.
-__device__ __forceinline__ float combine_row(const float2* __restrict__ p, int chunks, int rows)
+__device__ __forceinline__ float combine_row(const float2* p, int chunks, int rows)
 {
     float M = -INFINITY;
 #pragma unroll 8
@@ -1135,8 +1135,7 @@ __device__ __forceinline__ void epilogue_scores(const TcArgs& a, const Plan& pl,
 
 // Every unit's row normalisers (calls of many units: pass 2 would form a
 // unit's normalisers once per CTA that works on it).
-__global__ void window_combine_kernel(Shape s, int chunks, const float2* __restrict__ partial,
-                                      float* __restrict__ lse2)
+__global__ void window_combine_kernel(Shape s, int chunks, const float2* partial, float* lse2)
 {
     after_previous();
     const int u = blockIdx.x;
@@ -1148,7 +1147,7 @@ __global__ void window_combine_kernel(Shape s, int chunks, const float2* __restr
 // Row normalisers supplied by the caller's prefill attention: per (request,
 // layer) the natural-log LSE of each window row over the keys it sees,
 // [Hq][W] = [Hkv][G W] -> lse2 = LSE log2(e) + log2(G W).
-__global__ void lse_from_prefill_kernel(Shape s, LseTable t, float* __restrict__ lse2)
+__global__ void lse_from_prefill_kernel(Shape s, LseTable t, float* lse2)
 {
     after_previous();
     const int u = blockIdx.x;
