@@ -38,7 +38,9 @@
  * Ownership: the caller owns every tensor passed in or out.  The library
  * owns the context, its device scratch and the per-request state.  All calls
  * are asynchronous on the caller's CUDA stream (`bacon_stream` is a
- * cudaStream_t; NULL means the legacy default stream).  A call returns the
+ * cudaStream_t; NULL means the legacy default stream): a call's work starts
+ * after all earlier work of the stream, and later work starts after it,
+ * however the caller's own kernels are launched.  A call returns the
  * launch-time status; no exception crosses the ABI.  On error the message of
  * the failing call is available from bacon_last_error() on the same thread.
  *

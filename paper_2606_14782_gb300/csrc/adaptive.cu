@@ -144,7 +144,7 @@ adaptive_select_kernel(Shape s, int keep_window, AdaptArgs a)
 __global__ void __launch_bounds__(256)
 gather_flat_kernel(GatherTable tab, Shape s, const int32_t* counts, int* err)
 {
-    after_previous();
+    wait_previous();
     const int pair = blockIdx.y;
     const int total = tab.kept[pair];  // rows of the pair
     const int cpr = s.d / 8;

@@ -883,7 +883,7 @@ bacon_status bacon_compact(bacon_ctx* ctx, const void* k, const void* v, const i
     gt.vo[0] = static_cast<uint16_t*>(v_out);
     gt.idx[0] = idx;
     gt.kept[0] = count;
-    BACON_CUDA(launch_gather(gt, s, ctx->err, static_cast<cudaStream_t>(stream)), "gather launch");
+    BACON_CUDA(launch_gather(gt, s, ctx->err, static_cast<cudaStream_t>(stream), true), "gather launch");
     return BACON_OK;
 }
 

@@ -575,7 +575,8 @@ template <int T, int PER, bool ADAPT>
 __global__ void __launch_bounds__(T, 1024 / T)
 calibrate_select_kernel(Shape s, Calib c, CalibArgs a)
 {
-    after_previous();
+    wait_previous();
+    if (ADAPT || (a.compute_scores && a.do_select)) release_next();  // not the call's last
     const int u = blockIdx.x;
     calibrate_unit<T, PER, ADAPT>(s, c, a, u, a.lambda + u, a.idx[u / s.hkv]);
 }
@@ -636,7 +637,7 @@ calibrate_sweep_kernel(Shape s, CalibTable t, SweepArgs sw, CalibArgs a)
     __shared__ SelectScratch<T> sel_sm;
     __shared__ int ties[32], offsets[32];
     __shared__ float red_s[32], red_v[32];
-    after_previous();
+    wait_previous();
     const int u = blockIdx.x, j = blockIdx.y;
     const Calib& c = t.c[j];
     const int N = s.N, win = c.keep_window ? s.W : 0, n_cand = N - win;
@@ -707,7 +708,8 @@ cudaError_t launch_select_t(const Shape& s, const Calib& c, const CalibArgs& a, 
     cudaError_t e = cudaFuncSetAttribute(calibrate_select_kernel<T, PER, ADAPT>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
-    return launch_after(calibrate_select_kernel<T, PER, ADAPT>, s.units, T, sm, st, s, c, a);
+    return launch(!a.compute_scores, calibrate_select_kernel<T, PER, ADAPT>, s.units, T, sm, st, s,
+                  c, a);
 }
 
 template <int T, int PER>

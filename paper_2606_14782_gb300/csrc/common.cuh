@@ -74,18 +74,34 @@ __device__ __forceinline__ float key_float(uint32_t k)
 
 // ----------------------------------------------------------- launchers
 
-// Every kernel of the library is launched with programmatic stream
-// serialisation: its blocks may be placed while the previous kernel of the
-// stream finishes, and wait in after_previous() before they touch global
-// memory.  (griddepcontrol.wait returns once that kernel has completed and its
-// writes are visible.  Every block of every kernel waits, so completion is
-// transitive along the stream, and a kernel releases its successor's blocks
-// only after its own wait.)  28 layers of 6528 tokens one by one, five
-// launches each: 1.45 -> 1.13 ms; 28 layers x 4096 tokens at once, five
-// launches: 101 -> 93 us.
+// The kernels of one call overlap (programmatic stream serialisation): all but
+// the first are launched by launch_after, their blocks may be placed while the
+// kernel before them finishes, and wait before they touch global memory.
+// griddepcontrol.wait returns once that one kernel has completed and its
+// writes are visible; that all earlier work has completed too follows only
+// because every block of every kernel of the call waits, and because the first
+// kernel starts in plain stream order (launch_first).  Over a call's edges it
+// would not: a caller's kernel that was itself launched programmatically may
+// complete before the one in front of it, which wrote K.  For the same reason
+// the last kernel of a call releases nobody early (wait_previous alone), so
+// that a caller's kernel never runs beside one of the library's.
+// us a pass without any overlap, with it inside the calls, and over their edges
+// too: 28 layers of 6528 tokens one by one, three calls each, 1433, 1318 and
+// 1130; 28 layers x 4096 tokens in one call 101, 96.6 and 93.3; one layer of
+// 16384 tokens without a context 35.2, 29.1 and 27.5.
+__device__ __forceinline__ void wait_previous()
+{
+    asm volatile("griddepcontrol.wait;\n" ::: "memory");
+}
+// The next kernel's blocks may be placed once every block has got here.
+__device__ __forceinline__ void release_next()
+{
+    asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
+}
 __device__ __forceinline__ void after_previous()
 {
-    asm volatile("griddepcontrol.wait;\n griddepcontrol.launch_dependents;\n" ::: "memory");
+    wait_previous();
+    release_next();
 }
 
 // Piece q of a row of the caller's K or V through the read-only path: the one
@@ -101,8 +117,8 @@ __device__ __forceinline__ uint4 load_input(const uint16_t* row, int q)
 }
 
 template <typename... P, typename... A>
-cudaError_t launch_after(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
-                         const A&... args)
+cudaError_t launch(bool first, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem,
+                   cudaStream_t st, const A&... args)
 {
     cudaLaunchAttribute attr;
     attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -113,8 +129,21 @@ cudaError_t launch_after(void (*kernel)(P...), dim3 grid, dim3 block, size_t sme
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
     cfg.attrs = &attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = first ? 0 : 1;
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+// A call's first kernel, and one that follows another of the same call.
+template <typename... P, typename... A>
+cudaError_t launch_first(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                         const A&... args)
+{
+    return launch(true, kernel, grid, block, smem, st, args...);
+}
+template <typename... P, typename... A>
+cudaError_t launch_after(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                         const A&... args)
+{
+    return launch(false, kernel, grid, block, smem, st, args...);
 }
 
 // Calibration + selection per unit (Eqs. 5-17).  The residual of layer j of
@@ -145,7 +174,7 @@ struct CalibArgs {
     int taken_stride = 0;
     int guaranteed = 0;
     uint2* key_range = nullptr;
-    int compute_scores;  // 1: V, B~, lambda, S from B and the residuals
+    int compute_scores;  // 1: V, B~, lambda, S from B and the residuals; 0: the call's only kernel
     int do_select;       // 1: top-B selection into idx
     int write_S;
     int* err;
@@ -195,7 +224,9 @@ constexpr int kMaxAdaptive = 200 * 1024;
 cudaError_t launch_gather_flat(const GatherTable& tab, const Shape& s, const int32_t* counts,
                                int* err, cudaStream_t st);
 
-// Gather of the kept K/V rows (kept counts may differ between pairs).
-cudaError_t launch_gather(const GatherTable& tab, const Shape& s, int* err, cudaStream_t st);
+// Gather of the kept K/V rows (kept counts may differ between pairs); `first`:
+// nothing of the same call comes before it.
+cudaError_t launch_gather(const GatherTable& tab, const Shape& s, int* err, cudaStream_t st,
+                          bool first = false);
 
 }  // namespace bacon

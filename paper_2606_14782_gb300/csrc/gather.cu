@@ -11,7 +11,7 @@ namespace {
 __global__ void __launch_bounds__(256)
 gather_kernel(GatherTable tab, Shape s, int* err)
 {
-    after_previous();
+    wait_previous();
     const int u = blockIdx.y;
     const int pair = u / s.hkv, h = u - pair * s.hkv;
     const int kept = tab.kept[pair];
@@ -36,14 +36,14 @@ gather_kernel(GatherTable tab, Shape s, int* err)
 
 }  // namespace
 
-cudaError_t launch_gather(const GatherTable& tab, const Shape& s, int* err, cudaStream_t st)
+cudaError_t launch_gather(const GatherTable& tab, const Shape& s, int* err, cudaStream_t st, bool first)
 {
     int kept = 0;
     for (int p = 0; p < s.units / s.hkv; ++p) kept = tab.kept[p] > kept ? tab.kept[p] : kept;
     if (kept <= 0) return cudaSuccess;
     const int pieces = kept * (s.d / 8);
     dim3 grid((pieces + 255) / 256, s.units);
-    return launch_after(gather_kernel, grid, 256, 0, st, tab, s, err);
+    return launch(first, gather_kernel, grid, 256, 0, st, tab, s, err);
 }
 
 }  // namespace bacon

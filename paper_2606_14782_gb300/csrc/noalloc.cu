@@ -65,7 +65,7 @@ int take_fault()
 __global__ void __launch_bounds__(1024)
 poison_on_error_kernel(int* err, float* B, float* Q, float* E, size_t n)
 {
-    after_previous();
+    wait_previous();
     if (*reinterpret_cast<const volatile int*>(err) == 0) return;
     const float nan = __int_as_float(0x7fc00000);
     for (size_t i = threadIdx.x; i < n; i += blockDim.x) {

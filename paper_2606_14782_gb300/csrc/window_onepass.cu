@@ -452,7 +452,7 @@ cudaError_t launch_d(const TcArgs& a, const TcMaps& m, cudaStream_t st)
     if (e != cudaSuccess) return e;
     const int sms = num_sms_onepass();
     const int grid = a.s.units < sms ? a.s.units : sms;
-    return launch_after(window_onepass_kernel<D, SPEC>, grid, kThreads, bytes, st, a, m);
+    return launch_first(window_onepass_kernel<D, SPEC>, grid, kThreads, bytes, st, a, m);
 }
 
 }  // namespace

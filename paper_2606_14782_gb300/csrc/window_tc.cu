@@ -1403,7 +1403,7 @@ cudaError_t launch_impl(const TcArgs& args, const TcMaps& m, cudaStream_t st)
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
     if (e != cudaSuccess) return e;
     const int grid = a.items < sms ? a.items : sms;
-    return launch_after(window_tc_kernel<D, PASS>, grid, kThreads, bytes, st, a, pl, m);
+    return launch(PASS == 1, window_tc_kernel<D, PASS>, grid, kThreads, bytes, st, a, pl, m);
 }
 
 }  // namespace
@@ -1413,7 +1413,7 @@ int window_tc_max_rows() { return 512; }
 cudaError_t launch_lse_from_prefill(const Shape& s, const LseTable& t, float* lse2, cudaStream_t st)
 {
     const int threads = s.rows < 512 ? ((s.rows + 31) / 32) * 32 : 512;
-    return launch_after(lse_from_prefill_kernel, s.units, threads, 0, st, s, t, lse2);
+    return launch_first(lse_from_prefill_kernel, s.units, threads, 0, st, s, t, lse2);
 }
 
 cudaError_t launch_window_combine(const Shape& s, int chunks, const float2* partial,
