@@ -240,7 +240,9 @@ class Context:
         ix = [[torch.empty((self.kv_heads, kept[l]), dtype=torch.int32, device=k.device)
                for l in range(Ly)] for _ in range(R)]
         pairs = [(r, l) for r in range(R) for l in range(Ly)]
-        tq, tk, tv = (_pair_table(t, len(pairs)) if t.is_contiguous() else
+        # (a tensor of other requests or layers is indexed pair by pair)
+        tq, tk, tv = (_pair_table(t, len(pairs))
+                      if t.is_contiguous() and tuple(t.shape[:2]) == (R, Ly) else
                       _ptr_array([t[r, l].data_ptr() for r, l in pairs]) for t in (qwin, k, v))
         tko = _ptr_array([ko[r][l].data_ptr() for r, l in pairs])
         tvo = _ptr_array([vo[r][l].data_ptr() for r, l in pairs])
