@@ -582,6 +582,18 @@ const void* host_device_pointer(const void* p)
     return at.devicePointer;
 }
 
+// Whether p is memory of the context's device (not managed, the host's or
+// another device's).
+bool own_memory(const bacon_ctx* c, const void* p)
+{
+    cudaPointerAttributes at;
+    if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return at.type == cudaMemoryTypeDevice && at.device == c->device;
+}
+
 bacon_status check_pointer_arrays(const bacon_ctx* c, int pairs, const void* const* q,
                                   const void* const* k, const void* const* v, void* const* ko,
                                   void* const* vo)
@@ -817,9 +829,11 @@ bacon_status bacon_score_layer(bacon_ctx* ctx, bacon_state* st, int layer, const
     a.write_S = 1;
     a.err = ctx->err;
     // the caller's copy of S comes from the kernel too (28 layers x 6528
-    // tokens: 1.60 -> 1.49 ms without 28 copies) unless its rows are not aligned for
-    // the kernel's 16-byte stores
-    a.S_copy = scores_out && aligned16(scores_out) ? scores_out : nullptr;
+    // tokens: 1.60 -> 1.49 ms without 28 copies) when its rows are aligned for
+    // the kernel's 16-byte stores and lie in this device's own memory; the
+    // copy takes anything else that CUDA can address, or reports it
+    a.S_copy = scores_out && aligned16(scores_out) && own_memory(ctx, scores_out) ? scores_out
+                                                                                  : nullptr;
     BACON_CUDA(launch_calibrate_select(s, calib_of(ctx), a, cs), "calibrate launch");
     if (scores_out && !a.S_copy)
         BACON_CUDA(cudaMemcpyAsync(scores_out, st->S, sizeof(float) * ctx->hkv * seq_len,

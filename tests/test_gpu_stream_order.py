@@ -87,6 +87,32 @@ class Captured:
         self.do("cuGraphDestroy", self.graph)
 
 
+def test_scores_elsewhere_are_copied():
+    """A layer's scores go into the caller's device array from the kernel, and
+    into other memory (page-locked here) by a copy behind it."""
+    wl = workloads.CONFIGS["tiny"].with_(layers=1)
+    x = workloads.generate(wl, seed=5, device="cuda")
+    ctx = bacon.Context(1, wl.kv_heads, wl.q_heads, wl.head_dim, wl.window, wl.pool, 64,
+                        max_seq_len=wl.seq_len, max_requests=1)
+    state = bacon.State(ctx)
+    device = torch.empty(wl.kv_heads, wl.seq_len, device="cuda")
+    host = torch.empty(wl.kv_heads, wl.seq_len, pin_memory=True)
+    for out, copies in ((device, []), (host, [MEMCPY])):
+        def body():
+            state.reset()
+            return state.score_layer(0, x.qwin[0, 0], x.k[0, 0], scores_out=out)
+
+        g = Captured(body)
+        assert g.chain()[0] == [KERNEL] * 3 + copies
+        out.fill_(7)
+        torch.cuda.synchronize()
+        g.replay()
+        g.close()
+    assert torch.equal(host, device.cpu())
+    state.close()
+    ctx.close()
+
+
 GQA = dict(layers=3, q_heads=8, kv_heads=2, head_dim=128, seq_len=1200, visual=(16, 1100))
 ONE_PASS = dict(layers=3, q_heads=4, kv_heads=4, head_dim=64, seq_len=640)
 SWEEP = [dict(m=4), dict(m=2, r=3), dict(rho=1)]
