@@ -34,11 +34,17 @@ def _flags(extra=()):
              "-I", os.path.join(ROOT, "include")] + ARCH + list(extra))
 
 
+def inputs() -> list[str]:
+    """Every file the library is built from, the translation units first."""
+    return (sorted(glob.glob(os.path.join(CSRC, "*.cu")))
+            + sorted(p for ext in ("cuh", "h") for p in glob.glob(os.path.join(CSRC, "*." + ext)))
+            + [os.path.join(ROOT, "include", "bacon.h"), os.path.abspath(__file__)])
+
+
 def build(force: bool = False, verbose: bool = False, extra_flags=()) -> str:
     """Compile every CUDA translation unit and link libbacon.so; returns its path."""
-    sources = sorted(glob.glob(os.path.join(CSRC, "*.cu")))
-    headers = glob.glob(os.path.join(CSRC, "*.cuh")) + [os.path.join(ROOT, "include", "bacon.h")]
-    newest = max(os.path.getmtime(p) for p in sources + headers + [__file__])
+    sources = [p for p in inputs() if p.endswith(".cu")]
+    newest = max(os.path.getmtime(p) for p in inputs())
     if not force and os.path.exists(LIB) and os.path.getmtime(LIB) >= newest:
         return LIB
     os.makedirs(BUILD, exist_ok=True)
