@@ -78,6 +78,11 @@ __device__ __forceinline__ void load_run(const float* src, int i0, int n, float*
 // range narrows by another histogram) find their own rank: a thread counts
 // the gathered keys above and equal to its own, and the one whose ranks span
 // k publishes the result.  Six block barriers in the usual case.
+//
+// Ranges are compared by 32-bit differences from their lower end.  The bins
+// span at most 2^32 from the given range's lower end, so a top bin that
+// reaches past the largest word wraps to words below that end, where no
+// included key is.
 template <int T>
 struct SelectScratch {
     static constexpr int kBins = 4 * T;  // one 16-byte piece per thread
@@ -116,10 +121,11 @@ __device__ __forceinline__ void boundary_bin(SelectScratch<T>& sc, int remaining
 
 // each(f) calls f(included, key) for every element of the calling thread
 // (a flag instead of a branch around the call: the loads of a thread's
-// elements and their tests then overlap); 1 <= k <= the block's included keys; kmin / kmax: the thread's share of a key
-// range that holds all of them.  Every thread returns the same result.  The
-// scratch may be used again after the call's last barrier: a second call's
-// first writes touch only what no thread reads after that barrier.
+// elements and their tests then overlap); 1 <= k <= the block's included keys;
+// kmin / kmax: the thread's share of a key range that holds all of them.  Every
+// thread returns the same result.  The scratch may be used again after the
+// call's last barrier: a second call's first writes touch only what no thread
+// reads after that barrier.
 template <int T, typename EachFn>
 __device__ __forceinline__ SelectResult select_each(EachFn each, int k, SelectScratch<T>& sc,
                                                     uint32_t kmin, uint32_t kmax)
@@ -152,7 +158,7 @@ __device__ __forceinline__ SelectResult select_each(EachFn each, int k, SelectSc
         lo += (uint32_t)sc.out[0] << shift;
         remaining = sc.out[1];
         const int in_bin = sc.out[2];
-        last = min((1u << shift) - 1u, ~lo);  // (the top bin may reach past 2^32)
+        last = (1u << shift) - 1u;  // (the top bin may reach past 2^32, see above)
         if (shift == 0) return {lo, remaining, in_bin};
         if (in_bin <= S::kFew) break;
         // many keys in one bin (plateaus of equal scores): narrow the range
