@@ -47,7 +47,6 @@ bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) ==
 
 constexpr int kChunkTokens = 1024;  // pass-1 token chunk (multiple of the 128-token tile)
 constexpr size_t kLastBytes = 24ull << 20;  // host path: keys of the last pipelined part, at most
-constexpr int kMaxSeq = 24576;      // calibration keeps 2 x N fp32 in shared memory
 static_assert(kMaxVariants == BACON_MAX_VARIANTS, "variant table size");
 
 // Makes the context's device current for the duration of a call.
@@ -670,8 +669,8 @@ bacon_status bacon_init(bacon_ctx** out, int layers, int kv_heads, int q_heads, 
     if ((long long)prm.max_requests * layers > kMaxPairs)
         return fail(BACON_EINVAL, "max_requests * layers = %lld exceeds %d",
                     (long long)prm.max_requests * layers, kMaxPairs);
-    if (prm.max_seq_len < window || prm.max_seq_len > kMaxSeq)
-        return fail(BACON_EINVAL, "max_seq_len %d outside [window, %d]", prm.max_seq_len, kMaxSeq);
+    if (prm.max_seq_len < window || prm.max_seq_len > kMaxPrompt)
+        return fail(BACON_EINVAL, "max_seq_len %d outside [window, %d]", prm.max_seq_len, kMaxPrompt);
     const int group = q_heads / kv_heads;
     const int rows = group * window;
     if (rows > window_tc_max_rows())
@@ -1095,13 +1094,6 @@ bacon_status bacon_compress_host(bacon_ctx* ctx, int requests, const void* q_win
         BACON_CUDA(cudaStreamCreateWithFlags(&ctx->h2d, cudaStreamNonBlocking), "copy stream");
         BACON_CUDA(cudaStreamCreateWithFlags(&ctx->d2h, cudaStreamNonBlocking), "copy stream");
     }
-    while ((int)ctx->ev_in.size() < requests) {
-        cudaEvent_t a = nullptr, b = nullptr;
-        BACON_CUDA(cudaEventCreateWithFlags(&a, cudaEventDisableTiming), "event");
-        BACON_CUDA(cudaEventCreateWithFlags(&b, cudaEventDisableTiming), "event");
-        ctx->ev_in.push_back(a);
-        ctx->ev_done.push_back(b);
-    }
     // Parts are pipelined: every upload is queued on one copy stream, a part
     // is compressed on the caller's stream as soon as its inputs have landed
     // (layers in order: persistence reads the residuals of the layers
@@ -1197,7 +1189,6 @@ bacon_status bacon_compress_host(bacon_ctx* ctx, int requests, const void* q_win
                                    reinterpret_cast<char*>(ctx->hidx_buf) + i0, ib,
                                    cudaMemcpyDeviceToHost, ctx->d2h), "index download");
     }
-    (void)idx_count;
     // the error word comes with the outputs (the downloads follow every
     // kernel of the call); only a latched error takes the way of bacon_sync
     BACON_CUDA(cudaMemcpyAsync(ctx->h_err, ctx->err, sizeof(int), cudaMemcpyDeviceToHost, ctx->d2h),

@@ -17,8 +17,9 @@
 // ends), and position order is (thread, slot) order, so one block-wide
 // exclusive scan gives every thread its tie rank or its output offset.
 //
-// A unit is bound by latency: about 15 dependent rounds of a block barrier
-// each, one CTA per unit and at most one or two CTAs' worth of warps per SM.
+// A unit is bound by latency: 15 dependent rounds of a block barrier each (6
+// per selection, 2 sums, 1 scan; one more per selection whose last ties are
+// split), one CTA per unit and at most one or two CTAs' worth of warps per SM.
 // Keys in registers take the passes over all of them off shared memory, the
 // boundary bin's keys are ranked by counting instead of a second histogram
 // and a warp's sort, every warp finishes the block reductions itself (one
@@ -44,8 +45,7 @@ using namespace sel;
 // the same bits), sized so that threads x positions stays close to N: 8
 // positions per thread on 128, 256, 512 or 1024 threads up to 1024, 2048,
 // 4096 or 8192 tokens (several CTAs share an SM below 1024 threads), then
-// 1024 threads of 16 positions up to 16384 tokens and of 24 up to 24576.
-constexpr int kMaxPrompt = 24576;
+// 1024 threads of 16 positions up to 16384 tokens and of 24 up to kMaxPrompt.
 
 // Block-wide fp32 sums of NV values in one round, by a shuffle tree (pairwise,
 // so the rounding error grows with log2 of the count).  Every warp reduces
@@ -732,7 +732,8 @@ cudaError_t by_size(int N, F f)
     if (N <= 4096) return f.template run<512, 8>();
     if (N <= 8192) return f.template run<1024, 8>();
     if (N <= 16384) return f.template run<1024, 16>();
-    if (N <= kMaxPrompt) return f.template run<1024, 24>();
+    if (N <= 1024 * 24) return f.template run<1024, 24>();
+    static_assert(kMaxPrompt == 1024 * 24, "the largest size class");
     return cudaErrorInvalidValue;
 }
 

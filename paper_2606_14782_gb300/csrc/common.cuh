@@ -10,6 +10,10 @@ namespace bacon {
 // tensor pointers travel as kernel parameters.
 constexpr int kMaxPairs = 256;
 
+// Longest prompt: the calibration kernel's largest size class (1024 threads of
+// 24 positions).
+constexpr int kMaxPrompt = 1024 * 24;
+
 struct GatherTable {
     const uint16_t* k[kMaxPairs];
     const uint16_t* v[kMaxPairs];

@@ -177,7 +177,6 @@ __device__ __forceinline__ void fence_after_sync()
 {
     asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
 }
-__device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory"); }
 
 // 32 consecutive fp32 columns of this thread's TMEM lane.  The loads below
 // write float registers directly (a .b32 destination takes any 32-bit

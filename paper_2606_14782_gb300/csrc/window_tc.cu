@@ -202,9 +202,9 @@ __device__ __forceinline__ Segment segment_at(const TcArgs& a, const Plan& pl, i
 }
 
 // Jobs of one tile: the window rows, in 16-row granules, split into n_jobs
-// jobs of at most 128 rows (8 granules) as evenly as granules allow; job j
-// has n(j) rows starting at row0(j).  Pass 1 uses whole 128-row blocks
-// (8 granules per job).
+// jobs as evenly as granules allow; job j has n(j) rows starting at row0(j).
+// Pass 1 uses whole 128-row blocks (8 granules per job), pass 2 jobs of at most
+// 256 rows in two accumulators or 128 in four.
 struct JobTable {
     int n_jobs;
     int q, rem;  // granules per job, and how many jobs take one more
@@ -1351,11 +1351,11 @@ cudaError_t launch_impl(const TcArgs& args, const TcMaps& m, cudaStream_t st)
     const int rows = args.s.rows;
     const size_t budget = 227 * 1024 - 1024;
     // window rows in shared memory: whole 64-row TMA boxes.  Pass 1 runs
-    // whole 128-row MMA blocks over them in four 128-column accumulators; the
-    // last block's rows beyond q_rows read the next shared-memory region and
-    // their statistics are dropped (they are not window rows).  Pass 2 cuts
-    // the rows into jobs of up to 256 rows (two 256-column accumulators, the
-    // more efficient MMA shape) when shared memory allows, else up to 128.
+    // 128-row MMA blocks over them in four 128-column accumulators, a last block
+    // of one box as an M = 64 job; the statistics of a box's rows beyond the
+    // window rows are dropped.  Pass 2 cuts the rows into jobs of up to 256 rows
+    // (two 256-column accumulators, the more efficient MMA shape) when shared
+    // memory allows, else up to 128.
     Plan pl;
     pl.q_rows = (rows + kQBox - 1) / kQBox * kQBox;
     pl.last_m64 = (PASS == 1 && pl.q_rows % 128 == 64) ? 1 : 0;

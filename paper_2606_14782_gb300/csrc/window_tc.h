@@ -14,11 +14,12 @@ namespace bacon {
 // them all, and nothing has to be copied to the device before the launch.
 // Per pair it reads exactly what a map of that pair alone reads (rows beyond
 // the pair's own are zero).  A table of one map per pair has to be encoded and
-// copied first, and the next call waits for that copy: without it, 28 layers of a 6528-token prompt
-// scored one by one take 2.35 instead of 2.64 ms.  Pairs at uneven distances
-// take the table of one map each.  (The maps are a parameter of their own:
-// inside TcArgs, whose address would then escape, the window kernels spilled
-// and a 4 x 16384-token step took 1 % longer.)
+// copied first, and the next call waits for that copy: without it, 28 layers of
+// a 6528-token prompt scored one by one took 2.35 instead of 2.64 ms (before
+// the other changes to that path).  Pairs at uneven distances take the table of
+// one map each.  (The maps are a parameter of their own: inside TcArgs, whose
+// address would then escape, the window kernels spilled and a 4 x 16384-token
+// step took 1 % longer.)
 struct TcMaps {
     CUtensorMap k;  // [pairs][Hkv * N][d]
     CUtensorMap q;  // [pairs][Hq * W][d]
