@@ -11,8 +11,10 @@ one the waiter expects when the wait returns.  The model replays the
 kernels' sequence of waits and arrivals (TMA completions and MMA commits
 arrive asynchronously, commits in issue order) under random interleavings,
 on work lists cut the way the kernels cut them (each CTA a contiguous range
-of 1024-token chunks over (request, layer, kv-head) units), and checks that
-every schedule finishes and every wait returns in its own phase.  The
+over (request, layer, kv-head) units of 1024-token chunks, in pass 1 also of
+single row blocks of a chunk, or in pass 2 of 128-token tiles), and checks that
+every schedule finishes, every wait returns in its own phase and every MMA of
+pass 2 reads its own unit's bias.  The
 variant in which the merging group does not first wait for the slot's
 previous read (the kernels' earlier protocol) fails the check.  The one-pass
 kernel (logits resident in TMEM, two CTA-wide syncs per unit) is modelled
@@ -208,6 +210,18 @@ def cta_range(units, chunks_per_unit, total_ctas, cta):
     return [(g // chunks_per_unit, g % chunks_per_unit) for g in range(c0, c1)]
 
 
+def block_range(units, chunks_per_unit, blocks, total_ctas, cta):
+    """Pass 1 by row block of a chunk: the window rows change with every item."""
+    total = units * chunks_per_unit * blocks
+    g0, g1 = cta * total // total_ctas, (cta + 1) * total // total_ctas
+    out = []
+    for g in range(g0, g1):
+        c, rb = divmod(g, blocks)
+        u, ci = divmod(c, chunks_per_unit)
+        out.append((u * blocks + rb, ci))
+    return out
+
+
 def _cases(n=40, seed=3):
     rng = random.Random(seed)
     out = []
@@ -233,6 +247,37 @@ def test_pipeline_finishes_and_waits_in_phase(chunks, n_tiles, jobs, nbuf, stage
     for seed in range(6):
         fault = simulate(chunks, n_tiles, 8, jobs, nbuf, stages, q_slots, pass2, True, seed)
         assert fault is None, (seed, fault)
+
+
+def _tile_cases(n=24, seed=5):
+    rng = random.Random(seed)
+    out = []
+    while len(out) < n:
+        n_tiles = rng.choice([1, 2, 3, 5, 8, 11, 24])
+        units = rng.randint(1, 12)
+        ctas = rng.randint(1, units * n_tiles)
+        tiles = cta_range(units, n_tiles, ctas, rng.randrange(ctas))
+        if len(tiles) <= 40:
+            jobs, nbuf = rng.choice([(1, 4), (2, 2), (2, 4), (1, 2)])
+            out.append((tiles, n_tiles, jobs, nbuf, rng.choice([2, 3, 4]), rng.choice([1, 2])))
+    return out
+
+
+@pytest.mark.parametrize("tiles,n_tiles,jobs,nbuf,stages,q_slots", _tile_cases())
+def test_shares_of_tiles(tiles, n_tiles, jobs, nbuf, stages, q_slots):
+    for seed in range(6):
+        fault = simulate(tiles, n_tiles, 1, jobs, nbuf, stages, q_slots, True, True, seed)
+        assert fault is None, (seed, fault)
+
+
+@pytest.mark.parametrize("n_tiles,blocks,ctas", [(11, 2, 3), (16, 4, 5), (51, 4, 9), (8, 3, 2)])
+@pytest.mark.parametrize("q_slots", [1, 2])
+def test_shares_of_row_blocks(n_tiles, blocks, ctas, q_slots):
+    for cta in range(ctas):
+        items = block_range(2, -(-n_tiles // 8), blocks, ctas, cta)
+        for seed in range(3):
+            fault = simulate(items, n_tiles, 8, 1, 4, 3, q_slots, False, True, seed)
+            assert fault is None, (cta, seed, fault)
 
 
 def test_model_catches_the_unguarded_merger():
