@@ -612,8 +612,8 @@ def main():
         alt_ms = timed(alternate, args.steps, stream)
         line["fresh_buffers_each_step"] = {
             "ms_per_step": alt_ms, "extra_ms_per_step": alt_ms - ms,
-            "what": "two input sets in turn: every call encodes and uploads the TMA "
-                    "descriptors of its (request, layer) pairs"}
+            "what": "two input sets in turn: every call encodes the TMA descriptors of "
+                    "its tensors"}
         del x2, sets
 
     if not args.no_extras:
