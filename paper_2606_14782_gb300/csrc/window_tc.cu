@@ -1403,6 +1403,7 @@ cudaError_t launch_impl(const TcArgs& args, const TcMaps& m, cudaStream_t st)
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
     if (e != cudaSuccess) return e;
     const int grid = a.items < sms ? a.items : sms;
+    // (pass 1 is always its call's first kernel, pass 2 never is)
     return launch(PASS == 1, window_tc_kernel<D, PASS>, grid, kThreads, bytes, st, a, pl, m);
 }
 
